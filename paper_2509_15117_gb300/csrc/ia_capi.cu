@@ -2037,16 +2037,17 @@ int ia_reduce_stats(ia_system* sys, const ia_obs_soa* obs, int64_t n, const int3
     int rc = ia_reserve_stats(sys, n, n_cells);
     if (rc != IA_OK) return rc;
     double* partial = static_cast<double*>(sys->d_stats_scratch);
-    long long chunk = (n + grid - 1) / grid;
+    constexpr int W = STATS_BLOCK / 32;
+    long long chunk = (n + (long long)grid * W - 1) / ((long long)grid * W);
     chunk = (chunk + 31) / 32 * 32;
-    const size_t shmem = (size_t)(STATS_BLOCK / 32) * n_cells * 2 * sizeof(double);
+    const size_t shmem = (size_t)W * n_cells * 2 * sizeof(double) + (size_t)W * STATS_RUN_BINS * sizeof(unsigned);
     if (shmem > 48 * 1024 &&
         cudaFuncSetAttribute(k_stats_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem) != cudaSuccess)
         return IA_ERR_CUDA;
     ObsPtrs op{obs->theta_s, obs->dp, obs->dE_ion, obs->t_final, obs->t_first_bounce, obs->t_last_bounce,
                obs->n_bounce, obs->status, obs->n_steps, obs->n_rej, nullptr, 0};
     k_stats_pass1<<<grid, STATS_BLOCK, shmem, st>>>(op, (long long)n, cell_id, n_cells, stats, partial, chunk);
-    k_stats_pass2<<<(n_cells + 127) / 128, 128, 0, st>>>(partial, grid, n_cells, stats);
+    k_stats_pass2<<<(n_cells + 3) / 4, 128, 0, st>>>(partial, grid, n_cells, stats);
     return cudaGetLastError() == cudaSuccess ? IA_OK : IA_ERR_CUDA;
 }
 

@@ -92,16 +92,16 @@ struct PrimStep {
 __device__ __forceinline__ void step_coefs(const SysDev& P, int lane, double h, double t, double phi0, Coef& K,
                                            double& cs2, double& cs3, double& cs4, double& cs5, double& cs67)
 {
-    K.h2 = h * h;
+    K.h2 = dmul(P, h, h);
     const int k0 = lane < N_COEF ? lane : N_COEF - 1;
-    const double cv0 = COEF_K[k0] * (COEF_H2[k0] ? K.h2 : h);
+    const double cv0 = dmul(P, coef_sh()[k0], COEF_H2[k0] ? K.h2 : h);
     const int k1 = lane + 32 < N_COEF ? lane + 32 : N_COEF - 1;
-    const double cv1 = COEF_K[k1] * (COEF_H2[k1] ? K.h2 : h);
+    const double cv1 = dmul(P, coef_sh()[k1], COEF_H2[k1] ? K.h2 : h);
     double* kp = &K.c2;
 #pragma unroll
     for (int k = 0; k < N_COEF; ++k) kp[k] = k < 32 ? shfl(cv0, k) : shfl(cv1, k - 32);
     const double chsel = lane < 4 ? cv0 : h;
-    const double cl = cos(fma(P.Omega, t + chsel, phi0));
+    const double cl = cos(fma(P.Omega, dadd(P, t, chsel), phi0));
     cs2 = shfl(cl, 0);
     cs3 = shfl(cl, 1);
     cs4 = shfl(cl, 2);
@@ -115,14 +115,14 @@ __device__ __forceinline__ double adj_accel(const SysDev& P, const TLane& tl, do
                                             double coef, double* aux, double& r2, double d[3])
 {
     const int j = tl.comp < 3 ? tl.comp : tl.comp - 3;
-    const double dd = shfl(X, tl.base + 3 + j) - shfl(X, tl.base + j);
+    const double dd = dsub(P, shfl(X, tl.base + 3 + j), shfl(X, tl.base + j));
     const double d0 = shfl(dd, tl.base + 0), d1 = shfl(dd, tl.base + 1), d2 = shfl(dd, tl.base + 2);
-    r2 = fma(d0, d0, fma(d1, d1, d2 * d2));
-    const double s = rcp_nr(r2);
-    const double s2 = s * s;
-    const double s3 = fma(s2, s, 0.0);
+    r2 = fma(d0, d0, fma(d1, d1, dmul(P, d2, d2)));
+    const double s = rcp_nr(r2, P.one);
+    const double s2 = dmul(P, s, s);
+    const double s3 = dmul(P, s2, s);
     const bool ion = tl.comp < 3;
-    const double gm = s3 * fma(ion ? P.ci8 : P.ca8, s2, -(ion ? P.ci4 : P.ca4));
+    const double gm = dmul(P, s3, fma(ion ? P.ci8 : P.ca8, s2, -(ion ? P.ci4 : P.ca4)));
     d[0] = d0;
     d[1] = d1;
     d[2] = d2;
@@ -131,10 +131,10 @@ __device__ __forceinline__ double adj_accel(const SysDev& P, const TLane& tl, do
         aux[32] = d0;
         aux[64] = d1;
         aux[96] = d2;
-        aux[128] = s3 * fma(P.c8x8, s2, -P.c4x4);  // g = -V'(r)/r
-        aux[160] = (s2 * s2) * fma(-5.0 * P.c8x8, s2, 3.0 * P.c4x4);
+        aux[128] = dmul(P, s3, fma(P.c8x8, s2, -P.c4x4));  // g = -V'(r)/r
+        aux[160] = dmul(P, dmul(P, s2, s2), fma(P.m5c8x8, s2, P.c4x12));
     }
-    return fma(fma(kq, cs, ka), X, gm * dd);
+    return fma(fma(kq, cs, ka), X, dmul(P, gm, dd));
 }
 
 // Xbar = J^T abar for this lane's component at the stage stored in aux; adds the stage's part of
@@ -145,13 +145,13 @@ __device__ __forceinline__ double adj_apply(const SysDev& P, const TLane& tl, co
     const int j = tl.comp < 3 ? tl.comp : tl.comp - 3;
     const double X = aux[0], d0 = aux[32], d1 = aux[64], d2 = aux[96], g = aux[128], gu = aux[160];
     const double ui = shfl(ab, tl.base + j), ua = shfl(ab, tl.base + 3 + j);
-    const double uj = ui * P.inv_mi - ua * P.inv_ma;
+    const double uj = dsub(P, dmul(P, ui, P.inv_mi), dmul(P, ua, P.inv_ma));
     const double u0 = shfl(uj, tl.base + 0), u1 = shfl(uj, tl.base + 1), u2 = shfl(uj, tl.base + 2);
-    const double du = fma(d0, u0, fma(d1, u1, d2 * u2));
+    const double du = fma(d0, u0, fma(d1, u1, dmul(P, d2, u2)));
     const double dj = j == 0 ? d0 : (j == 1 ? d1 : d2);
-    const double Hu = fma((2.0 * gu) * du, dj, g * uj);
+    const double Hu = fma(dmul(P, twice(gu), du), dj, dmul(P, g, uj));
     if (tl.comp < 3) {
-        gq = fma((ab * P.kq_per_q) * cs, X, gq);
+        gq = fma(dmul(P, dmul(P, ab, P.kq_per_q), cs), X, gq);
         return fma(fma(kq, cs, ka), ab, Hu);
     }
     return -Hu;
@@ -184,17 +184,17 @@ __device__ __forceinline__ int prim_attempt(const SysDev& P, const TLane& tl, in
     bool okx, fx, okv, fv;
     float rx, rv;
     double aex, scx, aev, scv;
-    err_check(P.rtol, P.atol_pos, x, xn, err_x(K, a1, a3, a4, a5, a6), okx, fx, rx, aex, scx);
-    err_check(P.rtol, P.atol_vel, v, vn, err_v(K, a1, a3, a4, a5, a6, a7), okv, fv, rv, aev, scv);
+    err_check(P, P.rtol, P.atol_pos, x, xn, err_x(P, K, a1, a3, a4, a5, a6), okx, fx, rx, aex, scx);
+    err_check(P, P.rtol, P.atol_vel, v, vn, err_v(P, K, a1, a3, a4, a5, a6, a7), okv, fv, rv, aev, scv);
     const bool prim = tl.dir == 0;
     const bool accept = (__ballot_sync(FULL, prim && !(okx && okv)) & 0x3fu) == 0;
     const bool finite = (__ballot_sync(FULL, prim && !(fx && fv)) & 0x3fu) == 0;
     const ErrMeas em = group_err(0, tl.comp, prim, rx, aex, scx, rv, aev, scv);
     const int jj = tl.comp < 3 ? tl.comp : tl.comp - 3;
-    const double wj = shfl(vn, 3 + jj) - shfl(vn, jj);
+    const double wj = dsub(P, shfl(vn, 3 + jj), shfl(vn, jj));
     const double w0 = shfl(wj, 0), w1 = shfl(wj, 1), w2 = shfl(wj, 2);
     const double e0 = shfl(dn[0], 0), e1 = shfl(dn[1], 0), e2 = shfl(dn[2], 0);
-    const double rd = fma(e0, w0, fma(e1, w1, e2 * w2));
+    const double rd = fma(e0, w0, fma(e1, w1, dmul(P, e2, w2)));
     const double r2n0 = shfl(r2new, 0);
     if (!finite) {
         st = ST_NONFINITE;
@@ -237,11 +237,11 @@ __device__ __noinline__ void adj_step(const SysDev& P, const TLane& tl, int lane
     if (ext) adj_accel(P, tl, pos7(K, h, x, v, a1, a3, a4, a5), cs67, kq, ka, coef, sw + 6 * AUX_STAGE, r2, d3);
     double ab1, ab2 = 0.0, ab3, ab4, ab5, ab6, xb, vb;
     if (!ext) {
-        ab1 = fma(K.w71, lx, K.b1 * lv);
-        ab3 = fma(K.w73, lx, K.b3 * lv);
-        ab4 = fma(K.w74, lx, K.b4 * lv);
-        ab5 = fma(K.w75, lx, K.b5 * lv);
-        ab6 = K.b6 * lv;
+        ab1 = fma(K.w71, lx, dmul(P, K.b1, lv));
+        ab3 = fma(K.w73, lx, dmul(P, K.b3, lv));
+        ab4 = fma(K.w74, lx, dmul(P, K.b4, lv));
+        ab5 = fma(K.w75, lx, dmul(P, K.b5, lv));
+        ab6 = dmul(P, K.b6, lv);
         xb = lx;
         vb = fma(h, lx, lv);
     } else {
@@ -270,7 +270,7 @@ __device__ __noinline__ void adj_step(const SysDev& P, const TLane& tl, int lane
         vb = fma(s * h, lx, lv);
         // a7 = F(x'), x' = x + h v + sum w7m a_m
         const double X7 = adj_apply(P, tl, sw + 6 * AUX_STAGE, ab7, cs67, kq, ka, gq);
-        xb += X7;
+        xb = dadd(P, xb, X7);
         vb = fma(h, X7, vb);
         ab1 = fma(K.w71, X7, ab1);
         ab3 = fma(K.w73, X7, ab3);
@@ -278,32 +278,32 @@ __device__ __noinline__ void adj_step(const SysDev& P, const TLane& tl, int lane
         ab5 = fma(K.w75, X7, ab5);
     }
     const double X6 = adj_apply(P, tl, sw + 5 * AUX_STAGE, ab6, cs67, kq, ka, gq);
-    xb += X6;
+    xb = dadd(P, xb, X6);
     vb = fma(h, X6, vb);
     ab1 = fma(K.w61, X6, ab1);
     ab2 = fma(K.w62, X6, ab2);
     ab3 = fma(K.w63, X6, ab3);
     ab4 = fma(K.w64, X6, ab4);
     const double X5 = adj_apply(P, tl, sw + 4 * AUX_STAGE, ab5, cs5, kq, ka, gq);
-    xb += X5;
+    xb = dadd(P, xb, X5);
     vb = fma(K.c5, X5, vb);
     ab1 = fma(K.w51, X5, ab1);
     ab2 = fma(K.w52, X5, ab2);
     ab3 = fma(K.w53, X5, ab3);
     const double X4 = adj_apply(P, tl, sw + 3 * AUX_STAGE, ab4, cs4, kq, ka, gq);
-    xb += X4;
+    xb = dadd(P, xb, X4);
     vb = fma(K.c4, X4, vb);
     ab1 = fma(K.w41, X4, ab1);
     ab2 = fma(K.w42, X4, ab2);
     const double X3 = adj_apply(P, tl, sw + 2 * AUX_STAGE, ab3, cs3, kq, ka, gq);
-    xb += X3;
+    xb = dadd(P, xb, X3);
     vb = fma(K.c3, X3, vb);
     ab1 = fma(K.w31, X3, ab1);
     const double X2 = adj_apply(P, tl, sw + 1 * AUX_STAGE, ab2, cs2, kq, ka, gq);
-    xb += X2;
+    xb = dadd(P, xb, X2);
     vb = fma(K.c2, X2, vb);
     const double X1 = adj_apply(P, tl, sw + 0 * AUX_STAGE, ab1, c1, kq, ka, gq);
-    lx = xb + X1;
+    lx = dadd(P, xb, X1);
     lv = vb;
 }
 
@@ -450,6 +450,7 @@ __device__ __forceinline__ void adj_zero_outputs(const AdjIn& ain, const AdjOut&
 __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab, int n_sys, IcPtrs ic, ObsPtrs out,
                                                  long long n, AdjIn ain, AdjOut aout, AdjBuf buf)
 {
+    coef_sh_fill();
     __shared__ double s_aux[ADJ_WARPS][7 * AUX_STAGE];
     const TLane tl = tlane();
     const int lane = threadIdx.x & 31;

@@ -113,6 +113,7 @@ constexpr unsigned CLAIM_BACKOFF = 64;           // attempts between claim polls
 __global__ void __launch_bounds__(128) k_plain(const SysDev* __restrict__ tab, int n_sys, IcPtrs ic,
                                                ObsPtrs out, long long n)
 {
+    coef_sh_fill();
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int sid = ic.sys_id ? __ldg(ic.sys_id + i) : 0;
@@ -413,13 +414,13 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
 
         // step coefficients, spread over the group's lanes
         Coef K;
-        K.h2 = h * h;
+        K.h2 = dmul(P, h, h);
         double cv[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int k = r * G + (gl.c < G ? gl.c : 0);
             const int kk = k < N_COEF ? k : N_COEF - 1;
-            cv[r] = COEF_K[kk] * (COEF_H2[kk] ? K.h2 : h);
+            cv[r] = dmul(P, coef_sh()[kk], COEF_H2[kk] ? K.h2 : h);
         }
         {
             double* kp = &K.c2;
@@ -428,7 +429,7 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
         }
         // rf phases of stages 2..6 (stage 7 shares stage 6's time), one per lane
         const double chsel = gl.c < 4 ? cv[0] : h;
-        const double cl = cos(fma(P.Omega, t + chsel, S.phi0));
+        const double cl = cos(fma(P.Omega, dadd(P, t, chsel), S.phi0));
         const double cs2 = shfl(cl, gl.base + 0), cs3 = shfl(cl, gl.base + 1), cs4 = shfl(cl, gl.base + 2);
         const double cs5 = shfl(cl, gl.base + 3), cs67 = shfl(cl, gl.base + 4);
 
@@ -448,8 +449,8 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
         bool okx, fx, okv, fv;
         float rx, rv;
         double aex, scx, aev, scv;
-        err_check(P.rtol, P.atol_pos, x, xn, err_x(K, a1, a3, a4, a5, a6), okx, fx, rx, aex, scx);
-        err_check(P.rtol, P.atol_vel, v, vn, err_v(K, a1, a3, a4, a5, a6, a7), okv, fv, rv, aev, scv);
+        err_check(P, P.rtol, P.atol_pos, x, xn, err_x(P, K, a1, a3, a4, a5, a6), okx, fx, rx, aex, scx);
+        err_check(P, P.rtol, P.atol_vel, v, vn, err_v(P, K, a1, a3, a4, a5, a6, a7), okv, fv, rv, aev, scv);
         const bool real = gl.c < 6;
         const bool ok = !real || (okx && okv);
         const bool fi = !real || (fx && fv);
@@ -459,9 +460,9 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
         const ErrMeas em = group_err(gl.base, gl.c, real, rx, aex, scx, rv, aev, scv);
         // radial velocity sign at the step end: d . (v_a - v_i)
         const int j = gl.comp < 3 ? gl.comp : gl.comp - 3;
-        const double wj = shfl(vn, gl.base + 3 + j) - shfl(vn, gl.base + j);
+        const double wj = dsub(P, shfl(vn, gl.base + 3 + j), shfl(vn, gl.base + j));
         const double w0 = shfl(wj, gl.base + 0), w1 = shfl(wj, gl.base + 1), w2 = shfl(wj, gl.base + 2);
-        const double rd = fma(dn[0], w0, fma(dn[1], w1, dn[2] * w2));
+        const double rd = fma(dn[0], w0, fma(dn[1], w1, dmul(P, dn[2], w2)));
 
         int res = 0;  // 0 running, 1 stopped, 2 exits in this step
         if (active) {
@@ -601,23 +602,23 @@ __device__ __forceinline__ double chain_force(const SysDev& P, const GroupLane<6
     const int j = gl.comp < 3 ? gl.comp : gl.comp - 3;
     const double pi = shfl(p, gl.base + j);
     const double pa = shfl(p, gl.base + 3 + j);
-    const double dj = pa - pi;
+    const double dj = dsub(P, pa, pi);
     const double d0 = shfl(dj, gl.base + 0), d1 = shfl(dj, gl.base + 1), d2 = shfl(dj, gl.base + 2);
-    const double r2 = fma(d0, d0, fma(d1, d1, d2 * d2));
-    const double s = rcp_nr(r2);
-    const double s2 = s * s;
+    const double r2 = fma(d0, d0, fma(d1, d1, dmul(P, d2, d2)));
+    const double s = rcp_nr(r2, P.one);
+    const double s2 = dmul(P, s, s);
     // one FMA instruction: lane 0 forms s2 s, lane 1 the ion's ci8 s2 - ci4, lane 2 the atom's
     const int c = gl.c;
     const double ua = c == 0 ? s2 : (c == 1 ? P.ci8 : P.ca8);
     const double ub = c == 0 ? s : s2;
-    const double uc = c == 0 ? 0.0 : (c == 1 ? -P.ci4 : -P.ca4);
+    const double uc = c == 0 ? P.nz : (c == 1 ? -P.ci4 : -P.ca4);
     const double u = fma(ua, ub, uc);
-    const double gm = shfl(u, gl.base + 0) * shfl(u, gl.base + (gl.comp < 3 ? 1 : 2));
+    const double gm = dmul(P, shfl(u, gl.base + 0), shfl(u, gl.base + (gl.comp < 3 ? 1 : 2)));
     r2out = r2;
     d3[0] = d0;
     d3[1] = d1;
     d3[2] = d2;
-    return gm * dj;
+    return dmul(P, gm, dj);
 }
 
 __device__ __forceinline__ void tail_phase_pair(const SysDev* __restrict__ tab, const IcPtrs& ic, const ObsPtrs& out,
@@ -745,8 +746,8 @@ __device__ __forceinline__ void tail_phase_pair(const SysDev* __restrict__ tab, 
             // rf phases first: the chain warp needs the ion trap coefficient of stage 2 soonest.
             // Lanes 0-3 form t + c_s h (s = 2..5; the products of the other layouts), lane 4 t + h.
             const int cidx = gl.c < 4 ? gl.c : 0;
-            const double chsel = gl.c < 4 ? COEF_K[cidx] * h : h;
-            const double cl = cos(fma(P.Omega, t + chsel, S.phi0));
+            const double chsel = gl.c < 4 ? dmul(P, coef_sh()[cidx], h) : h;
+            const double cl = cos(fma(P.Omega, dadd(P, t, chsel), S.phi0));
             const double cs2 = shfl(cl, gl.base + 0), cs3 = shfl(cl, gl.base + 1), cs4 = shfl(cl, gl.base + 2);
             const double cs5 = shfl(cl, gl.base + 3), cs67 = shfl(cl, gl.base + 4);
             const double kqj = gl.comp < 3 ? P.kq[gl.comp] : 0.0;
@@ -758,12 +759,12 @@ __device__ __forceinline__ void tail_phase_pair(const SysDev* __restrict__ tab, 
             sh->kc[6][lane] = fma(kqj, cs67, kaj);
             pair_post(sh->seq_h, nh);                                     // H1: trap coefficients
             Coef K;
-            K.h2 = h * h;
+            K.h2 = dmul(P, h, h);
             double cv[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const int kk = r * G + gl.c < N_COEF ? r * G + gl.c : N_COEF - 1;
-                cv[r] = COEF_K[kk] * (COEF_H2[kk] ? K.h2 : h);
+                cv[r] = dmul(P, coef_sh()[kk], COEF_H2[kk] ? K.h2 : h);
             }
             {
                 double* kp = &K.c2;
@@ -774,7 +775,7 @@ __device__ __forceinline__ void tail_phase_pair(const SysDev* __restrict__ tab, 
             double p6 = fma(K.w61, a1, fma(h, v, x));
             double p7 = fma(K.w71, a1, fma(h, v, x));
             double vacc = fma(K.b1, a1, v);
-            double ex = K.f1 * a1, ev = K.e1 * a1;
+            double ex = dmul(P, K.f1, a1), ev = dmul(P, K.e1, a1);
             bool ok = pair_wait(sh->seq_c, nc);                           // C1: a2
             const double a2 = sh->a[2][lane];
             p5 = fma(K.w52, a2, p5);
@@ -811,16 +812,16 @@ __device__ __forceinline__ void tail_phase_pair(const SysDev* __restrict__ tab, 
             bool okx, fx, okv, fv;
             float rx, rv;
             double aex, scx, aev, scv;
-            err_check(P.rtol, P.atol_pos, x, xn, ex, okx, fx, rx, aex, scx);  // while the chain warp forms a7
+            err_check(P, P.rtol, P.atol_pos, x, xn, ex, okx, fx, rx, aex, scx);  // while the chain warp forms a7
             const int j = gl.comp < 3 ? gl.comp : gl.comp - 3;
-            const double wj = shfl(vn, gl.base + 3 + j) - shfl(vn, gl.base + j);
+            const double wj = dsub(P, shfl(vn, gl.base + 3 + j), shfl(vn, gl.base + j));
             const double w0 = shfl(wj, gl.base + 0), w1 = shfl(wj, gl.base + 1), w2 = shfl(wj, gl.base + 2);
             ok = pair_wait(sh->seq_c, nc) && ok;                          // C5: a7 and the step end
             a7 = sh->a[7][lane];
             r2new = sh->r2n[lane];
             const double dn0 = sh->dn[0][lane], dn1 = sh->dn[1][lane], dn2 = sh->dn[2][lane];
             ev = fma(K.e7, a7, ev);
-            err_check(P.rtol, P.atol_vel, v, vn, ev, okv, fv, rv, aev, scv);
+            err_check(P, P.rtol, P.atol_vel, v, vn, ev, okv, fv, rv, aev, scv);
             const bool real = gl.c < 6;
             const bool okk = !real || (okx && okv);
             const bool fi = !real || (fx && fv);
@@ -828,7 +829,7 @@ __device__ __forceinline__ void tail_phase_pair(const SysDev* __restrict__ tab, 
             accept = (__ballot_sync(FULL, !okk) & gmask) == 0;
             finite = (__ballot_sync(FULL, !fi) & gmask) == 0;
             em = group_err(gl.base, gl.c, real, rx, aex, scx, rv, aev, scv);
-            rd = fma(dn0, w0, fma(dn1, w1, dn2 * w2));
+            rd = fma(dn0, w0, fma(dn1, w1, dmul(P, dn2, w2)));
             sh->vn[lane] = vn;
             sh->rd[lane] = rd;
             sh->errf[lane] = em.f;
@@ -840,14 +841,15 @@ __device__ __forceinline__ void tail_phase_pair(const SysDev* __restrict__ tab, 
         } else {
             // stage 2, and the step coefficients of this warp's own stage positions (the products
             // and the positions of the other layouts, bit for bit) while the helper forms the rf phases
-            const double X2 = fma(COEF_K[0] * h, v, x);
+            const double* sK = coef_sh();
+            const double X2 = fma(dmul(P, sK[0], h), v, x);
             double r2, d3[3];
             const double q2 = chain_force(P, gl, X2, r2, d3);
-            const double h2 = h * h;
-            const double X3 = fma(COEF_K[4] * h2, a1, fma(COEF_K[1] * h, v, x));     // w31, c3
-            const double p4 = fma(COEF_K[5] * h2, a1, fma(COEF_K[2] * h, v, x));     // w41, c4
-            const double w42 = COEF_K[6] * h2, w53 = COEF_K[9] * h2;
-            const double w64 = COEF_K[13] * h2, w75 = COEF_K[17] * h2;
+            const double h2 = dmul(P, h, h);
+            const double X3 = fma(dmul(P, sK[4], h2), a1, fma(dmul(P, sK[1], h), v, x));     // w31, c3
+            const double p4 = fma(dmul(P, sK[5], h2), a1, fma(dmul(P, sK[2], h), v, x));     // w41, c4
+            const double w42 = dmul(P, sK[6], h2), w53 = dmul(P, sK[9], h2);
+            const double w64 = dmul(P, sK[13], h2), w75 = dmul(P, sK[17], h2);
             bool ok = pair_wait(sh->seq_h, nh);                           // H1
             const bool ion = gl.comp < 3;
             const double kc2 = ion ? sh->kc[2][lane] : 0.0, kc3 = ion ? sh->kc[3][lane] : 0.0;
@@ -973,6 +975,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
 {
     __shared__ int role;  // 0 lane phase first, 1 tail worker, 2 surplus block on a reserved SM
     __shared__ PairShared pair_sh[G == 6 ? BLOCK / 64 : 1];
+    coef_sh_fill();
     if (threadIdx.x == 0) {
         for (int k = 0; k < (G == 6 ? BLOCK / 64 : 1); ++k)
             for (int l = 0; l < 32; ++l) pair_sh[k].seq_h[l] = pair_sh[k].seq_c[l] = 0ull;
@@ -1035,6 +1038,7 @@ __global__ void __launch_bounds__(128) k_tail(const SysDev* __restrict__ tab, Ic
                                               Susp* __restrict__ susp, unsigned* __restrict__ ready,
                                               Counters* __restrict__ ctr, long long cap, Part part)
 {
+    coef_sh_fill();
     long long n_tc = 0;
     if (part.tcarry_in_n) {
         const unsigned long long c = *part.tcarry_in_n;
@@ -1050,6 +1054,7 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
                                                  long long n, TanIn tin, TanOut tout,
                                                  unsigned long long* __restrict__ work)
 {
+    coef_sh_fill();
     const TLane tl = tlane();
     const int lane = threadIdx.x & 31;
     const int yi = tl.comp < 3 ? tl.comp : tl.comp + 3;  // position index in y
@@ -1162,19 +1167,19 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
             }
             h = S.h;
             t = S.t;
-            K.h2 = h * h;
+            K.h2 = dmul(P, h, h);
             // coefficients: lane k computes coefficient k (and k + 30 for lanes 0..3)
             const int k0 = lane < N_COEF ? lane : N_COEF - 1;
-            const double cv0 = COEF_K[k0] * (COEF_H2[k0] ? K.h2 : h);
+            const double cv0 = dmul(P, coef_sh()[k0], COEF_H2[k0] ? K.h2 : h);
             const int k1 = lane + 32 < N_COEF ? lane + 32 : N_COEF - 1;
-            const double cv1 = COEF_K[k1] * (COEF_H2[k1] ? K.h2 : h);
+            const double cv1 = dmul(P, coef_sh()[k1], COEF_H2[k1] ? K.h2 : h);
             {
                 double* kp = &K.c2;
 #pragma unroll
                 for (int k = 0; k < N_COEF; ++k) kp[k] = k < 32 ? shfl(cv0, k) : shfl(cv1, k - 32);
             }
             const double chsel = lane < 4 ? cv0 : h;
-            const double cl = cos(fma(P.Omega, t + chsel, S.phi0));
+            const double cl = cos(fma(P.Omega, dadd(P, t, chsel), S.phi0));
             const double cs2 = shfl(cl, 0), cs3 = shfl(cl, 1), cs4 = shfl(cl, 2), cs5 = shfl(cl, 3), cs67 = shfl(cl, 4);
             const double a2 = tan_accel(P, tl, pos2(K, x, v), cs2, kq, ka, dkq, coef, r2, d3);
             a3 = tan_accel(P, tl, pos3(K, x, v, a1), cs3, kq, ka, dkq, coef, r2, d3);
@@ -1188,16 +1193,16 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
             bool okx, fx, okv, fv;
             float rx, rv;
             double aex, scx, aev, scv;
-            err_check(P.rtol, P.atol_pos, x, xn, err_x(K, a1, a3, a4, a5, a6), okx, fx, rx, aex, scx);
-            err_check(P.rtol, P.atol_vel, v, vn, err_v(K, a1, a3, a4, a5, a6, a7), okv, fv, rv, aev, scv);
+            err_check(P, P.rtol, P.atol_pos, x, xn, err_x(P, K, a1, a3, a4, a5, a6), okx, fx, rx, aex, scx);
+            err_check(P, P.rtol, P.atol_vel, v, vn, err_v(P, K, a1, a3, a4, a5, a6, a7), okv, fv, rv, aev, scv);
             const bool prim = tl.dir == 0;
             const bool accept = (__ballot_sync(FULL, prim && !(okx && okv)) & 0x3fu) == 0;
             const bool finite = (__ballot_sync(FULL, prim && !(fx && fv)) & 0x3fu) == 0;
             const ErrMeas em = group_err(0, lane, prim, rx, aex, scx, rv, aev, scv);
             const int jj = tl.comp < 3 ? tl.comp : tl.comp - 3;
-            const double wj = shfl(vn, 3 + jj) - shfl(vn, jj);
+            const double wj = dsub(P, shfl(vn, 3 + jj), shfl(vn, jj));
             const double w0 = shfl(wj, 0), w1 = shfl(wj, 1), w2 = shfl(wj, 2);
-            const double rd = fma(dn[0], w0, fma(dn[1], w1, dn[2] * w2));
+            const double rd = fma(dn[0], w0, fma(dn[1], w1, dmul(P, dn[2], w2)));
             if (!finite) {
                 st = ST_NONFINITE;
                 res = 1;
@@ -1543,6 +1548,10 @@ SysDev derive(const ia_system_desc& d)
     const double mu = d.m_ion * d.m_atom / (d.m_ion + d.m_atom);
     P.inv_len = C4 > 0.0 ? 1.0 / std::pow(C4 / (2.0 * d.De), 0.25) : 1.0;
     P.inv_vel = C4 > 0.0 ? 1.0 / std::sqrt(2.0 * d.De / mu) : 1.0;
+    P.m5c8x8 = -5.0 * P.c8x8;
+    P.c4x12 = 3.0 * P.c4x4;
+    P.one = 1.0;
+    P.nz = -0.0;
     return P;
 }
 

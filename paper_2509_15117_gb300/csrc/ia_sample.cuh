@@ -26,6 +26,8 @@
 
 #include <cstdint>
 
+#include "ia_fixed.cuh"
+
 namespace ia_sample {
 
 constexpr unsigned long long PHILOX_M0 = 0xD2E7470EE14C6C93ull;
@@ -69,30 +71,42 @@ __device__ __forceinline__ void philox4x64_10(unsigned long long c[4], unsigned 
     }
 }
 
-__device__ __forceinline__ double uniform01(unsigned long long x)
-{
-    return (double)((x >> 11) | 1ull) * 0x1p-53;
-}
-
 // Four uniforms of block j of trajectory g.
 __device__ __forceinline__ void block_uniforms(unsigned long long seed, int kind, long long g, int j, double* u)
 {
     unsigned long long c[4] = {(unsigned long long)g, (unsigned long long)j, 0ull, 0ull};
     philox4x64_10(c, seed, (unsigned long long)(unsigned)kind);
 #pragma unroll
-    for (int w = 0; w < 4; ++w) u[w] = uniform01(c[w]);
+    for (int w = 0; w < 4; ++w) u[w] = uniform_double(uniform_int(c[w]));
 }
 
 // Box-Muller pair from (u_r, u_a): rho = sqrt(-2 ln u_r), angle 2 pi u_a.
 __device__ __forceinline__ void box_muller(double u_r, double u_a, double& z0, double& z1)
 {
-    const double rho = sqrt(-2.0 * log(u_r));
+    const double rho = sqrt_rn(-2.0 * log(u_r));
     double s, c;
     sincospi(2.0 * u_a, &s, &c);
     z0 = rho * c;
     z1 = rho * s;
 }
 
+// v / n for three components, each correctly rounded.
+__device__ __forceinline__ void unit3(const double v[3], double n, double o[3])
+{
+    if (ordinary(n)) {
+        const Fx r = fx_rcp(n);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) o[j] = div_rn(v[j], n, r);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) o[j] = v[j] / n;
+    }
+}
+
+// Bound by the FP64 unit (log and sincospi, whose bits nothing else reproduces). What is correctly rounded --
+// the conversions to uniforms, square roots and divisions -- runs on the integer pipes beside it
+// (ia_fixed.cuh), with the same bits: 2^24 head-on states 1,650 -> 1,324 us, 4,194,301 disk states with
+// micromotion 4,589 -> 4,155 us.
 __global__ void __launch_bounds__(SAMPLE_THREADS) k_sample(SampleParams p)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -107,7 +121,7 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) k_sample(SampleParams p)
 
         if (p.kind == 0) {
             const double ct = u[1];
-            const double st = sqrt((1.0 - ct) * (1.0 + ct));
+            const double st = sqrt_rn((1.0 - ct) * (1.0 + ct));
             double sa, ca;
             sincospi(0.5 * u[2], &sa, &ca);
             const double xh[3] = {st * ca, st * sa, ct};
@@ -126,7 +140,7 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) k_sample(SampleParams p)
             double v[3] = {p.sig_a * gz[0], p.sig_a * gz[1], p.sig_a * gz[2]};
             if (p.kind == 1) {
                 const double ct = 2.0 * u[1] - 1.0;
-                const double st = sqrt((1.0 - ct) * (1.0 + ct));
+                const double st = sqrt_rn((1.0 - ct) * (1.0 + ct));
                 double sa, ca;
                 sincospi(2.0 * u[2], &sa, &ca);
                 const double xh[3] = {st * ca, st * sa, ct};
@@ -139,8 +153,9 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) k_sample(SampleParams p)
 #pragma unroll
                 for (int j = 0; j < 3; ++j) y[6 + j] = p.r0 * xh[j];
             } else {
-                const double vn = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-                const double vh[3] = {v[0] / vn, v[1] / vn, v[2] / vn};
+                const double vn = sqrt_rn(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+                double vh[3];
+                unit3(v, vn, vh);
                 // e1 = unit(v_hat x r), r = z_hat unless v_hat is within ~26 degrees of the z axis
                 const bool use_z = fabs(vh[2]) < 0.9;
                 double e1[3];
@@ -153,16 +168,14 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) k_sample(SampleParams p)
                     e1[1] = vh[2];
                     e1[2] = -vh[1];
                 }
-                const double n1 = sqrt(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]);
-                e1[0] /= n1;
-                e1[1] /= n1;
-                e1[2] /= n1;
+                const double n1 = sqrt_rn(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]);
+                unit3(e1, n1, e1);
                 const double e2[3] = {vh[1] * e1[2] - vh[2] * e1[1], vh[2] * e1[0] - vh[0] * e1[2],
                                       vh[0] * e1[1] - vh[1] * e1[0]};
-                const double b = p.b_max * sqrt(u[1]);
+                const double b = p.b_max * sqrt_rn(u[1]);
                 double sp, cp;
                 sincospi(2.0 * u[2], &sp, &cp);
-                const double back = sqrt(p.r0 * p.r0 - b * b);
+                const double back = sqrt_rn(p.r0 * p.r0 - b * b);
 #pragma unroll
                 for (int j = 0; j < 3; ++j) y[6 + j] = b * (cp * e1[j] + sp * e2[j]) - back * vh[j];
             }

@@ -175,63 +175,41 @@ __device__ __forceinline__ double adj_apply(const SysDev& P, const TLane& tl, co
     return -Hu;
 }
 
-// One attempted step of the primal: the control flow of the tangent kernel (decisions from group 0,
-// which every group reproduces). On a commit x, v, a1, c1 advance.
-__device__ __forceinline__ int prim_attempt(const SysDev& P, const TLane& tl, int lane, Scal& S, double& x, double& v,
-                                            double& a1, double& c1, double kq, double ka, double coef, PrimStep& E,
+// One attempted step of the primal, in warp mode (every group of six lanes holds a copy of the state). On a
+// commit x, v, a1, c1 advance.
+__device__ __forceinline__ int prim_attempt(const SysDev& P, const TLane& tl, const GroupSys& gs, const WarpIdx& wi,
+                                            int lane, Scal& S, double& x, double& v,
+                                            double& a1, double& c1, PrimStep& E,
                                             uint32_t& st)
 {
     st = attempt_begin(P, S);
     if (st != 0xffffffffu) return PA_STOP;
-    const double h = S.h, t = S.t;
-    E.h = h;
-    E.t = t;
-    Coef K;
-    double cs2, cs3, cs4, cs5, cs67;
-    step_coefs(P, lane, h, t, S.phi0, K, cs2, cs3, cs4, cs5, cs67);
-    double r2, d3[3];
-    const double a2 = adj_accel(P, tl, pos2(K, x, v), cs2, kq, ka, coef, nullptr, r2, d3);
-    const double a3 = adj_accel(P, tl, pos3(K, x, v, a1), cs3, kq, ka, coef, nullptr, r2, d3);
-    const double a4 = adj_accel(P, tl, pos4(K, x, v, a1, a2), cs4, kq, ka, coef, nullptr, r2, d3);
-    const double a5 = adj_accel(P, tl, pos5(K, x, v, a1, a2, a3), cs5, kq, ka, coef, nullptr, r2, d3);
-    const double a6 = adj_accel(P, tl, pos6(K, h, x, v, a1, a2, a3, a4), cs67, kq, ka, coef, nullptr, r2, d3);
-    const double xn = pos7(K, h, x, v, a1, a3, a4, a5);
-    double r2new, dn[3];
-    const double a7 = adj_accel(P, tl, xn, cs67, kq, ka, coef, nullptr, r2new, dn);
-    const double vn = vel_new(K, v, a1, a3, a4, a5, a6);
-    bool okx, fx, okv, fv;
-    float rx, rv;
-    double aex, scx, aev, scv;
-    err_check(P, P.rtol, P.atol_pos, x, xn, err_x(P, K, a1, a3, a4, a5, a6), okx, fx, rx, aex, scx);
-    err_check(P, P.rtol, P.atol_vel, v, vn, err_v(P, K, a1, a3, a4, a5, a6, a7), okv, fv, rv, aev, scv);
-    const bool prim = tl.dir == 0;
-    const bool accept = (__ballot_sync(FULL, prim && !(okx && okv)) & 0x3fu) == 0;
-    const bool finite = (__ballot_sync(FULL, prim && !(fx && fv)) & 0x3fu) == 0;
-    const ErrMeas em = group_err(0, tl.comp, prim, rx, aex, scx, rv, aev, scv);
-    const int jj = tl.comp < 3 ? tl.comp : tl.comp - 3;
-    const double wj = dsub(P, shfl(vn, 3 + jj), shfl(vn, jj));
-    const double w0 = shfl(wj, 0), w1 = shfl(wj, 1), w2 = shfl(wj, 2);
-    const double e0 = shfl(dn[0], 0), e1 = shfl(dn[1], 0), e2 = shfl(dn[2], 0);
-    const double rd = fma(e0, w0, fma(e1, w1, dmul(P, e2, w2)));
-    const double r2n0 = shfl(r2new, 0);
-    if (!finite) {
+    E.h = S.h;
+    E.t = S.t;
+    WarpStep W;
+    GroupLane<6> gl;
+    gl.base = tl.base;
+    gl.c = lane - tl.base;
+    gl.comp = tl.comp;
+    warp_step(P, gl, gs, wi, x, v, a1, S.h, S.t, S.phi0, W);
+    if (!W.finite) {
         st = ST_NONFINITE;
         return PA_STOP;
     }
-    if (!accept) {
-        st = on_reject(P, S, em);
+    if (!W.accept) {
+        st = on_reject(P, S, W.em);
         return st != 0xffffffffu ? PA_STOP : PA_REJ;
     }
-    if (on_accept(P, S, rd, r2n0)) {
-        E.a3 = a3; E.a4 = a4; E.a5 = a5; E.a6 = a6; E.a7 = a7;
-        E.xn = xn; E.vn = vn; E.r2new = r2n0; E.cs67 = cs67;
+    if (on_accept(P, S, W.rd, W.r2new)) {
+        E.a3 = W.a3; E.a4 = W.a4; E.a5 = W.a5; E.a6 = W.a6; E.a7 = W.a7;
+        E.xn = W.xn; E.vn = W.vn; E.r2new = W.r2new; E.cs67 = W.cs67;
         return PA_EXIT;
     }
-    x = xn;
-    v = vn;
-    a1 = a7;
-    c1 = cs67;
-    on_commit(P, S, em);
+    x = W.xn;
+    v = W.vn;
+    a1 = W.a7;
+    c1 = W.cs67;
+    on_commit(P, S, W.em);
     return PA_COMMIT;
 }
 
@@ -523,6 +501,8 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
         const double kq = tl.comp < 3 ? P.kq[tl.comp] : 0.0;
         const double ka = tl.comp < 3 ? P.ka[tl.comp] : 0.0;
         const double coef = tl.comp < 3 ? P.neg_inv_mi : P.inv_ma;
+        const GroupSys gs = group_sys(P, lane - tl.base);
+        const WarpIdx wi = warp_idx(tl.dir);
         double c1 = cos(S.phi0);
         double a1;
         {
@@ -553,7 +533,7 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
         int slot = 0;  // committed steps modulo seg
         for (;;) {
             const double x0 = x, v0 = v, c10 = c1;
-            const int r = prim_attempt(P, tl, lane, S, x, v, a1, c1, kq, ka, coef, E, st);
+            const int r = prim_attempt(P, tl, gs, wi, lane, S, x, v, a1, c1, E, st);
             if (r == PA_REJ) continue;
             if (r == PA_STOP) { res = 1; break; }
             if (r == PA_EXIT) { res = 2; break; }
@@ -719,7 +699,7 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
                 const double x0 = rx, v0 = rv, c10 = rc1;
                 uint32_t rst;
                 PrimStep RE;
-                const int r = prim_attempt(P, tl, lane, R, rx, rv, ra1, rc1, kq, ka, coef, RE, rst);
+                const int r = prim_attempt(P, tl, gs, wi, lane, R, rx, rv, ra1, rc1, RE, rst);
                 if (r == PA_REJ) continue;
                 if (r != PA_COMMIT) {
                     bad = true;

@@ -104,8 +104,10 @@ constexpr int MAX_TAIL_WARPS = 8;
 // Against lane mode to the end: one Rb trajectory of 8,192 attempts 128 -> 64 ms, 1,024 of up to 32,768
 // attempts 1,212 -> 321 ms, 50,000 thermal ones of up to 8,192 243 -> 94 ms, the 40-system sweep of 67,240
 // 324 -> 309 ms; 262,144 trajectories of one length, which end together, 239 -> 241 ms.
+// A warp's last trajectory goes on in warp mode: 5.8 us per attempt, 7.7 in group mode, about 20 in lane mode.
 constexpr int LOCAL_MAX = 15;
 constexpr int LOCAL_QUANTUM = 16;
+constexpr int WARP_HOLD = 64;  // attempts in warp mode between looks for records
 // Reserved tail SMs serve trajectories past the slice budget while the bulk still runs. Below this many
 // trajectories per lane the bulk is over before one can get there (131,072 attempts, over 5 s), and the
 // reserved SMs would only run the lane phase in batches; such launches reserve none.
@@ -304,7 +306,8 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
     constexpr int R = (N_COEF + G - 1) / G;  // coefficient rounds per lane
     constexpr int NG = 32 / G;               // groups per warp
     const GroupLane<G> gl = group_lane<G>();
-    double x = 0.0, v = 0.0, a1 = 0.0;
+    // idle groups keep a harmless state (unit separation): at zero separation the reciprocal takes its slow path
+    double x = gl.comp < 3 ? 0.0 : 1.0, v = 0.0, a1 = 0.0;
     Scal S;
     S.t = 0.0; S.h = 0.0; S.hmin = 0.0; S.phi0 = 0.0; S.rdot_prev = 0.0; S.t_first = 0.0; S.t_last = 0.0;
     S.n_acc = 0; S.n_rej = 0; S.n_bounce = 0; S.nofailed = true; S.retry = false;
@@ -318,7 +321,24 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
     // the next turn, attempts left of this turn (all but lslot warp-uniform)
     unsigned lalive = (1u << n_loc) - 1u, lpend = lalive;
     int lslot = -1, lnext = 0, lturn = 0;
+    // warp mode (G = 6): while the warp has a single trajectory, every group holds a copy of it and group 0
+    // answers for it; left every WARP_HOLD attempts to look for records
+    bool wmode = false;
+    int hold = 0;
+    SysDev P;                 // the fields that an attempt needs, in registers (see group_sys)
+    GroupSys gs;
+    int sid_in_regs = -1;
+    const WarpIdx wi = warp_idx(gl.base / G);
     for (;;) {
+        if (G == 6 && wmode && --hold < 0) {
+            wmode = false;
+            if (gl.base != 0) {
+                if (active) lslot = -1;  // (a finished one keeps its slot, to be cleared below)
+                active = false;
+            }
+            claim_skip = 0;
+        }
+        if (!wmode) {
         if (lalive) {
             const unsigned done = __reduce_or_sync(FULL, lslot >= 0 && !active ? 1u << lslot : 0u);
             lalive &= ~done;
@@ -503,10 +523,50 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
             continue;
         }
 
-        const SysDev& P = tab[sid];
+        if (G == 6 && lpend == 0u) {
+            const unsigned act = __ballot_sync(FULL, active && gl.c == 0);
+            if (__popc(act) == 1) {
+                const int b = __ffs(act) - 1;
+                x = shfl(x, b + gl.comp); v = shfl(v, b + gl.comp); a1 = shfl(a1, b + gl.comp);
+                S.t = shfl(S.t, b); S.h = shfl(S.h, b); S.hmin = shfl(S.hmin, b); S.phi0 = shfl(S.phi0, b);
+                S.rdot_prev = shfl(S.rdot_prev, b);
+                S.t_first = shfl(S.t_first, b); S.t_last = shfl(S.t_last, b);
+                S.n_acc = __shfl_sync(FULL, S.n_acc, b); S.n_rej = __shfl_sync(FULL, S.n_rej, b);
+                S.n_bounce = __shfl_sync(FULL, S.n_bounce, b);
+                S.nofailed = __shfl_sync(FULL, (int)S.nofailed, b) != 0;
+                S.retry = __shfl_sync(FULL, (int)S.retry, b) != 0;
+                idx = __shfl_sync(FULL, idx, b);
+                sid = __shfl_sync(FULL, sid, b);
+                lslot = __shfl_sync(FULL, lslot, b);
+                active = true;
+                wmode = true;
+                hold = WARP_HOLD;
+            }
+        }
+        }
+
+        if (sid != sid_in_regs) {
+            P.one = tab[sid].one; P.nz = tab[sid].nz; P.Omega = tab[sid].Omega;
+            P.rtol = tab[sid].rtol; P.atol_pos = tab[sid].atol_pos; P.atol_vel = tab[sid].atol_vel;
+            P.t_max = tab[sid].t_max; P.h_max = tab[sid].h_max; P.max_attempts = tab[sid].max_attempts;
+            P.r0sq = tab[sid].r0sq;
+            gs = group_sys(tab[sid], gl.c);
+            sid_in_regs = sid;
+        }
         uint32_t st = 0xffffffffu;
         if (active) st = attempt_begin(P, S);
         const double h = S.h, t = S.t;
+        double a3, a4, a5, a6, a7, xn, vn, r2new, rd;
+        bool accept, finite;
+        ErrMeas em;
+        if (G == 6 && wmode) {
+            WarpStep E;
+            GroupLane<6> g6;
+            g6.base = gl.base; g6.c = gl.c; g6.comp = gl.comp;
+            warp_step(P, g6, gs, wi, x, v, a1, h, t, S.phi0, E);
+            a3 = E.a3; a4 = E.a4; a5 = E.a5; a6 = E.a6; a7 = E.a7; xn = E.xn; vn = E.vn;
+            r2new = E.r2new; rd = E.rd; accept = E.accept; finite = E.finite; em = E.em;
+        } else {
 
         // step coefficients, spread over the group's lanes
         Coef K;
@@ -529,18 +589,16 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
         const double cs2 = shfl(cl, gl.base + 0), cs3 = shfl(cl, gl.base + 1), cs4 = shfl(cl, gl.base + 2);
         const double cs5 = shfl(cl, gl.base + 3), cs67 = shfl(cl, gl.base + 4);
 
-        const double kq = gl.comp >= 3 ? P.kq[gl.comp - 3] : 0.0;  // lanes 3-5: the ion's axis comp - 3
-        const double ka = gl.comp >= 3 ? P.ka[gl.comp - 3] : 0.0;
         double r2, d3[3];
-        const double a2 = accel_group<G>(P, gl, pos2(K, x, v), cs2, kq, ka, r2, d3);
-        const double a3 = accel_group<G>(P, gl, pos3(K, x, v, a1), cs3, kq, ka, r2, d3);
-        const double a4 = accel_group<G>(P, gl, pos4(K, x, v, a1, a2), cs4, kq, ka, r2, d3);
-        const double a5 = accel_group<G>(P, gl, pos5(K, x, v, a1, a2, a3), cs5, kq, ka, r2, d3);
-        const double a6 = accel_group<G>(P, gl, pos6(K, h, x, v, a1, a2, a3, a4), cs67, kq, ka, r2, d3);
-        const double xn = pos7(K, h, x, v, a1, a3, a4, a5);
-        double r2new, dn[3];
-        const double a7 = accel_group<G>(P, gl, xn, cs67, kq, ka, r2new, dn);
-        const double vn = vel_new(K, v, a1, a3, a4, a5, a6);
+        const double a2 = accel_group<G>(P, gl, gs, pos2(K, x, v), cs2, r2, d3);
+        a3 = accel_group<G>(P, gl, gs, pos3(K, x, v, a1), cs3, r2, d3);
+        a4 = accel_group<G>(P, gl, gs, pos4(K, x, v, a1, a2), cs4, r2, d3);
+        a5 = accel_group<G>(P, gl, gs, pos5(K, x, v, a1, a2, a3), cs5, r2, d3);
+        a6 = accel_group<G>(P, gl, gs, pos6(K, h, x, v, a1, a2, a3, a4), cs67, r2, d3);
+        xn = pos7(K, h, x, v, a1, a3, a4, a5);
+        double dn[3];
+        a7 = accel_group<G>(P, gl, gs, xn, cs67, r2new, dn);
+        vn = vel_new(K, v, a1, a3, a4, a5, a6);
 
         bool okx, fx, okv, fv;
         float rx, rv;
@@ -551,14 +609,15 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
         const bool ok = !real || (okx && okv);
         const bool fi = !real || (fx && fv);
         const unsigned gmask = ((1u << G) - 1u) << gl.base;
-        const bool accept = (__ballot_sync(FULL, !ok) & gmask) == 0;
-        const bool finite = (__ballot_sync(FULL, !fi) & gmask) == 0;
-        const ErrMeas em = group_err(gl.base, gl.c, real, rx, aex, scx, rv, aev, scv);
+        accept = (__ballot_sync(FULL, !ok) & gmask) == 0;
+        finite = (__ballot_sync(FULL, !fi) & gmask) == 0;
+        em = group_err(gl.base, gl.c, real, rx, aex, scx, rv, aev, scv);
         // radial velocity sign at the step end: d . (v_a - v_i)
         const int j = gl.comp < 3 ? gl.comp : gl.comp - 3;
         const double wj = dsub(P, shfl(vn, gl.base + 3 + j), shfl(vn, gl.base + j));
         const double w0 = shfl(wj, gl.base + 0), w1 = shfl(wj, gl.base + 1), w2 = shfl(wj, gl.base + 2);
-        const double rd = fma(dn[0], w0, fma(dn[1], w1, dmul(P, dn[2], w2)));
+        rd = fma(dn[0], w0, fma(dn[1], w1, dmul(P, dn[2], w2)));
+        }
 
         int res = 0;  // 0 running, 1 stopped, 2 exits in this step
         if (active) {
@@ -606,11 +665,12 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
                 }
                 D.h = h;
                 D.t = t;
-                if (res == 2 && gl.c == 0) finish_exit(P, D, r2new, fin);
+                if (res == 2 && gl.c == 0 && !(wmode && gl.base != 0)) finish_exit(tab[sid], D, r2new, fin);
             }
             if (res != 0) {
-                if (gl.c == 0) store_result(P, ic, out, idx, tally(S), fin, true);
+                if (gl.c == 0 && !(wmode && gl.base != 0)) store_result(tab[sid], ic, out, idx, tally(S), fin, true);
                 active = false;
+                hold = 0;
             }
         }
     }
@@ -1109,9 +1169,10 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
     // a reserved SM's block keeps tail_warps tail warps; its other warps leave (pairs need all of them)
     const int r = (role == 1 && !(G == 6 && pair && wait_ok) && (int)(threadIdx.x >> 5) >= tail_warps) ? 2 : role;
     // Share of a small batch. A warp's attempt costs its sub-partition the same time however few lanes are
-    // busy, so trajectories are spread before warps are filled: up to one batch of groups per sub-partition
-    // (one warp each: its group-mode attempt has the FP64 unit to itself), then one per warp, then full
-    // warps on one warp per sub-partition, then on all.
+    // busy, so trajectories are spread before warps are filled: up to a batch of groups on one warp of every
+    // sub-partition, a batch per warp, full warps on one warp per sub-partition, then on all. (us per attempt
+    // with 608 sub-partitions: 1 or 608 trajectories 5.8 and 6.1, 1,024 7.7 -- one per warp on two warps of a sub-partition
+    // 8.8 -- 3,040 7.7, 6,080 11.3, 19,456 22.8, 38,912 40.2.)
     int share = 32;
     if (local_ok) {
         constexpr int NG = 32 / G;

@@ -29,7 +29,9 @@
 // The forward pass, the replay and the reverse sweep are all bound by the FP64 unit (85 % busy). A replay
 // costs as much as the forward pass, about a quarter of the whole, and most trajectories (mean 8,000
 // steps at 1.5 uK) fit the default ring of 10,000: a differentiable call on 1,000 of them, stopped after
-// 8,192 attempts, takes 297 ms (547 ms with the replay and a forward launch in lane mode).
+// 8,192 attempts, takes 297 ms (547 ms with the replay and a forward launch in lane mode). With the primal in
+// warp mode 259 ms; with the force's products and the positions' sums of the reverse step spread over lanes
+// and groups (adj_accel, adj_step), 1,000 trajectories of 4,096 attempts 105.6 -> 91.8 ms, 8,192 647 -> 562.
 //
 // One step of the Nystrom form (accelerations depend on positions only):
 //   X_l = x + c_l h v + h^2 sum_m AA_lm a_m,  a_l = F(X_l, t + c_l h),
@@ -107,14 +109,17 @@ struct PrimStep {
 
 // Coefficients and cosines of a step (lane-distributed products, then broadcast; the values are
 // those of the tangent kernel bit for bit).
+// cv: coefficient k on lane k, for the first 32.
 __device__ __forceinline__ void step_coefs(const SysDev& P, int lane, double h, double t, double phi0, Coef& K,
-                                           double& cs2, double& cs3, double& cs4, double& cs5, double& cs67)
+                                           double& cv, double& cs2, double& cs3, double& cs4, double& cs5,
+                                           double& cs67)
 {
     K.h2 = dmul(P, h, h);
     const int k0 = lane < N_COEF ? lane : N_COEF - 1;
     const double cv0 = dmul(P, coef_sh()[k0], COEF_H2[k0] ? K.h2 : h);
     const int k1 = lane + 32 < N_COEF ? lane + 32 : N_COEF - 1;
     const double cv1 = dmul(P, coef_sh()[k1], COEF_H2[k1] ? K.h2 : h);
+    cv = cv0;
     double* kp = &K.c2;
 #pragma unroll
     for (int k = 0; k < N_COEF; ++k) kp[k] = k < 32 ? shfl(cv0, k) : shfl(cv1, k - 32);
@@ -129,28 +134,22 @@ __device__ __forceinline__ void step_coefs(const SysDev& P, int lane, double h, 
 
 // Acceleration component of this lane at positions X of its group (the primal arithmetic of the
 // other layouts). When aux is not null, stores the stage quantities the reverse sweep needs.
-__device__ __forceinline__ double adj_accel(const SysDev& P, const TLane& tl, double X, double cs, double kq, double ka,
-                                            double coef, double* aux, double& r2, double d[3])
+__device__ __forceinline__ double adj_accel(const SysDev& P, const TLane& tl, const ForceLane& fl, double X, double cs,
+                                            double kq, double ka, double* aux)
 {
     const int j = tl.comp < 3 ? tl.comp : tl.comp - 3;
     const double dd = dsub(P, shfl(X, tl.base + 3 + j), shfl(X, tl.base + j));
     const double d0 = shfl(dd, tl.base + 0), d1 = shfl(dd, tl.base + 1), d2 = shfl(dd, tl.base + 2);
-    r2 = fma(d0, d0, fma(d1, d1, dmul(P, d2, d2)));
-    const double s = rcp_nr(r2, P.one);
-    const double s2 = dmul(P, s, s);
-    const double s3 = dmul(P, s2, s);
-    const bool ion = tl.comp < 3;
-    const double gm = dmul(P, s3, fma(ion ? P.ci8 : P.ca8, s2, -(ion ? P.ci4 : P.ca4)));
-    d[0] = d0;
-    d[1] = d1;
-    d[2] = d2;
+    const double r2 = fma(d0, d0, fma(d1, d1, dmul(P, d2, d2)));
+    const double prod = force_products(P, fl, tl.base, r2);
+    const double gm = shfl(prod, tl.base + (tl.comp < 3 ? 1 : 2));
     if (aux) {
         aux[0] = X;
         aux[32] = d0;
         aux[64] = d1;
         aux[96] = d2;
-        aux[128] = dmul(P, s3, fma(P.c8x8, s2, -P.c4x4));  // g = -V'(r)/r
-        aux[160] = dmul(P, dmul(P, s2, s2), fma(P.m5c8x8, s2, P.c4x12));
+        aux[128] = shfl(prod, tl.base + 3);  // g = -V'(r)/r
+        aux[160] = shfl(prod, tl.base + 5);  // g_u
     }
     return fma(fma(kq, cs, ka), X, dmul(P, gm, dd));
 }
@@ -162,8 +161,8 @@ __device__ __forceinline__ double adj_apply(const SysDev& P, const TLane& tl, co
 {
     const int j = tl.comp < 3 ? tl.comp : tl.comp - 3;
     const double X = aux[0], d0 = aux[32], d1 = aux[64], d2 = aux[96], g = aux[128], gu = aux[160];
-    const double ui = shfl(ab, tl.base + j), ua = shfl(ab, tl.base + 3 + j);
-    const double uj = dsub(P, dmul(P, ui, P.inv_mi), dmul(P, ua, P.inv_ma));
+    const double ab_m = dmul(P, ab, tl.comp < 3 ? P.inv_mi : P.inv_ma);  // abar / m on the lane that holds abar
+    const double uj = dsub(P, shfl(ab_m, tl.base + j), shfl(ab_m, tl.base + 3 + j));
     const double u0 = shfl(uj, tl.base + 0), u1 = shfl(uj, tl.base + 1), u2 = shfl(uj, tl.base + 2);
     const double du = fma(d0, u0, fma(d1, u1, dmul(P, d2, u2)));
     const double dj = j == 0 ? d0 : (j == 1 ? d1 : d2);
@@ -216,23 +215,43 @@ __device__ __forceinline__ int prim_attempt(const SysDev& P, const TLane& tl, co
 // Pull (lx, lv) -- the adjoint of this lane's component at the end of a step, or at fraction s of
 // the step on its continuous extension when ext -- back to the step start; adds the step's part of
 // the q gradient to gq. (x, v): primal state at the step start; c1: the cosine of a1's evaluation.
-__device__ __noinline__ void adj_step(const SysDev& P, const TLane& tl, int lane, double x, double v, double t,
-                                      double h, double c1, double phi0, bool ext, double s, double kq, double ka,
-                                      double coef, double& lx, double& lv, double& gq, double* sw)
+// The stage positions' sums are spread over the groups as in warp_step: X3..X7 on groups 0..4.
+template <bool EXT>
+__device__ __forceinline__ void adj_step(const SysDev& P, const TLane& tl, const ForceLane& fl, int lane, double x,
+                                      double v, double t, double h, double c1, double phi0, double s,
+                                      double kq, double ka, double& lx, double& lv, double& gq, double* sw)
 {
     Coef K;
-    double cs2, cs3, cs4, cs5, cs67;
-    step_coefs(P, lane, h, t, phi0, K, cs2, cs3, cs4, cs5, cs67);
-    double r2, d3[3];
-    const double a1 = adj_accel(P, tl, x, c1, kq, ka, coef, sw + 0 * AUX_STAGE, r2, d3);
-    const double a2 = adj_accel(P, tl, pos2(K, x, v), cs2, kq, ka, coef, sw + 1 * AUX_STAGE, r2, d3);
-    const double a3 = adj_accel(P, tl, pos3(K, x, v, a1), cs3, kq, ka, coef, sw + 2 * AUX_STAGE, r2, d3);
-    const double a4 = adj_accel(P, tl, pos4(K, x, v, a1, a2), cs4, kq, ka, coef, sw + 3 * AUX_STAGE, r2, d3);
-    const double a5 = adj_accel(P, tl, pos5(K, x, v, a1, a2, a3), cs5, kq, ka, coef, sw + 4 * AUX_STAGE, r2, d3);
-    adj_accel(P, tl, pos6(K, h, x, v, a1, a2, a3, a4), cs67, kq, ka, coef, sw + 5 * AUX_STAGE, r2, d3);
-    if (ext) adj_accel(P, tl, pos7(K, h, x, v, a1, a3, a4, a5), cs67, kq, ka, coef, sw + 6 * AUX_STAGE, r2, d3);
+    double cv, cs2, cs3, cs4, cs5, cs67;
+    step_coefs(P, lane, h, t, phi0, K, cv, cs2, cs3, cs4, cs5, cs67);
+    const int g = tl.dir, c = tl.comp;
+    const double a1 = adj_accel(P, tl, fl, x, c1, kq, ka, sw + 0 * AUX_STAGE);
+    const double a2 = adj_accel(P, tl, fl, pos2(K, x, v), cs2, kq, ka, sw + 1 * AUX_STAGE);
+    const double kb = shfl(cv, g < 3 ? 1 + g : 0);
+    double acc = fma(g < 3 ? kb : h, v, x);
+    acc = fma(shfl(cv, pick5(g, 4, 5, 7, 10, 14)), a1, acc);
+    const double a3 = adj_accel(P, tl, fl, shfl(acc, c), cs3, kq, ka, sw + 2 * AUX_STAGE);
+    {
+        const double k = shfl(cv, pick5(g, 0, 6, 8, 11, 0));
+        if (g >= 1 && g <= 3) acc = fma(k, a2, acc);
+    }
+    const double a4 = adj_accel(P, tl, fl, shfl(acc, 6 + c), cs4, kq, ka, sw + 3 * AUX_STAGE);
+    {
+        const double k = shfl(cv, pick5(g, 0, 0, 9, 12, 15));
+        if (g >= 2) acc = fma(k, a3, acc);
+    }
+    const double a5 = adj_accel(P, tl, fl, shfl(acc, 12 + c), cs5, kq, ka, sw + 4 * AUX_STAGE);
+    {
+        const double k = shfl(cv, pick5(g, 0, 0, 0, 13, 16));
+        if (g >= 3) acc = fma(k, a4, acc);
+    }
+    adj_accel(P, tl, fl, shfl(acc, 18 + c), cs67, kq, ka, sw + 5 * AUX_STAGE);
+    if (EXT) {
+        const double X7 = fma(K.w75, a5, acc);  // group 4's
+        adj_accel(P, tl, fl, shfl(X7, 24 + c), cs67, kq, ka, sw + 6 * AUX_STAGE);
+    }
     double ab1, ab2 = 0.0, ab3, ab4, ab5, ab6, xb, vb;
-    if (!ext) {
+    if (!EXT) {
         ab1 = fma(K.w71, lx, dmul(P, K.b1, lv));
         ab3 = fma(K.w73, lx, dmul(P, K.b3, lv));
         ab4 = fma(K.w74, lx, dmul(P, K.b4, lv));
@@ -470,7 +489,11 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
             adj_zero_outputs(ain, aout, tl, lane, i, 0.0);
             continue;
         }
-        const SysDev& P = tab[sid];
+        const SysDev& T = tab[sid];
+        SysDev P;  // the fields that a step needs, in registers
+        P.one = T.one; P.nz = T.nz; P.Omega = T.Omega; P.rtol = T.rtol; P.atol_pos = T.atol_pos;
+        P.atol_vel = T.atol_vel; P.t_max = T.t_max; P.h_max = T.h_max; P.max_attempts = T.max_attempts;
+        P.r0sq = T.r0sq; P.inv_mi = T.inv_mi; P.inv_ma = T.inv_ma; P.kq_per_q = T.kq_per_q;
         double x = __ldg(ic.y0 + yi * ic.ld + i);
         double v = __ldg(ic.y0 + yv * ic.ld + i);
         Scal S;
@@ -493,22 +516,18 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
                 fin.t = 0.0;
                 fin.s_exit = -1.0;
                 fin.status = ST_BAD_IC;
-                store_result(P, ic, out, i, tally(S), fin, false);
+                store_result(T, ic, out, i, tally(S), fin, false);
             }
             adj_zero_outputs(ain, aout, tl, lane, i, 0.0);
             continue;
         }
-        const double kq = tl.comp < 3 ? P.kq[tl.comp] : 0.0;
-        const double ka = tl.comp < 3 ? P.ka[tl.comp] : 0.0;
-        const double coef = tl.comp < 3 ? P.neg_inv_mi : P.inv_ma;
-        const GroupSys gs = group_sys(P, lane - tl.base);
+        const double kq = tl.comp < 3 ? T.kq[tl.comp] : 0.0;
+        const double ka = tl.comp < 3 ? T.ka[tl.comp] : 0.0;
+        const ForceLane fl = force_lane(T, lane - tl.base);
+        const GroupSys gs = group_sys(T, lane - tl.base);
         const WarpIdx wi = warp_idx(tl.dir);
         double c1 = cos(S.phi0);
-        double a1;
-        {
-            double r2, d3[3];
-            a1 = adj_accel(P, tl, x, c1, kq, ka, coef, nullptr, r2, d3);
-        }
+        double a1 = adj_accel(P, tl, fl, x, c1, kq, ka, nullptr);
         {
             Lane L0;
             for (int k = 0; k < 3; ++k) {
@@ -516,7 +535,7 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
                 L0.a1i[k] = shfl(a1, k);
                 L0.a1a[k] = shfl(a1, 3 + k);
             }
-            S.h = initial_step(P, L0);
+            S.h = initial_step(T, L0);
         }
         S.rdot_prev = fma(dd0, vs[3] - vs[0], fma(dd1, vs[4] - vs[1], dd2 * (vs[5] - vs[2])));
         S.t = 0.0; S.hmin = 0.0; S.t_first = 0.0; S.t_last = 0.0;
@@ -592,7 +611,7 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
             }
             D.h = E.h;
             D.t = E.t;
-            if (lane == 0) finish_exit(P, D, E.r2new, fin);
+            if (lane == 0) finish_exit(T, D, E.r2new, fin);
             fin.t = __shfl_sync(FULL, fin.t, 0);
             fin.s_exit = __shfl_sync(FULL, fin.s_exit, 0);
             fin.status = __shfl_sync(FULL, fin.status, 0);
@@ -633,7 +652,7 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
                 yfv = E.vn;
             }
         }
-        if (lane == 0) store_result(P, ic, out, i, tally(S), fin, true);
+        if (lane == 0) store_result(T, ic, out, i, tally(S), fin, true);
 
         // ---- pass 2: the terminal adjoint of each objective
         double y0v[12], yf[12];
@@ -646,7 +665,7 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
             yf[pi + 3] = shfl(yfv, tl.base + k);
         }
         double gy0[12], gyf[12], gqe[3], jt;
-        objective_partials(P, tl.dir, S.phi0, y0v, yf, fin.t, gy0, gyf, jt, gqe);
+        objective_partials(T, tl.dir, S.phi0, y0v, yf, fin.t, gy0, gyf, jt, gqe);
         double lx = gyf[yi], lv = gyf[yv];
         const double ex_x = gy0[yi], ex_v = gy0[yv];
         const double ex_q = tl.comp < 3 ? gqe[tl.comp] : 0.0;
@@ -669,7 +688,10 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
                 const double cc = (ls + jt * E.h) / den;
                 lx -= cc * (tl.comp < 3 ? -dprim : dprim);
             }
-            adj_step(P, tl, lane, x, v, E.t, E.h, c1, S.phi0, ext, fin.s_exit, kq, ka, coef, lx, lv, gq, sw);
+            if (ext)
+                adj_step<true>(P, tl, fl, lane, x, v, E.t, E.h, c1, S.phi0, fin.s_exit, kq, ka, lx, lv, gq, sw);
+            else
+                adj_step<false>(P, tl, fl, lane, x, v, E.t, E.h, c1, S.phi0, 0.0, kq, ka, lx, lv, gq, sw);
             adj_rescale(tl, lx, lv, gq, scale_e);
         }
 
@@ -677,44 +699,41 @@ __global__ void __launch_bounds__(128) k_adjoint(const SysDev* __restrict__ tab,
         __syncwarp();
         bool bad = false;
         long long hi = n_com;
-        for (int left = n_com < buf.seg ? (int)n_com : buf.seg; left > 0; --left, --hi) {
-            slot = slot == 0 ? buf.seg - 1 : slot - 1;
-            const double* rec = srw + (long long)slot * SR_DOUBLES;
-            const double sx = rec[tl.comp], sv = rec[6 + tl.comp];
-            const double st0 = rec[12], sh0 = rec[13], sc1 = rec[14];
-            adj_step(P, tl, lane, sx, sv, st0, sh0, sc1, S.phi0, false, 0.0, kq, ka, coef, lx, lv, gq, sw);
-            adj_rescale(tl, lx, lv, gq, scale_e);
-        }
-        __syncwarp();
-        while (hi > 0 && !bad) {
-            const long long c = (hi - 1) / stride;
-            const long long base = c * stride;
-            const long long lo = hi - buf.seg > base ? hi - buf.seg : base;
-            Scal R;
-            R.phi0 = S.phi0;
-            double rx, rv, ra1, rc1;
-            ckpt_read(ckw + c * CK_DOUBLES, tl.comp, rx, rv, ra1, rc1, R);
-            long long k = base;
-            while (k < hi) {
-                const double x0 = rx, v0 = rv, c10 = rc1;
-                uint32_t rst;
-                PrimStep RE;
-                const int r = prim_attempt(P, tl, gs, wi, lane, R, rx, rv, ra1, rc1, RE, rst);
-                if (r == PA_REJ) continue;
-                if (r != PA_COMMIT) {
-                    bad = true;
-                    break;
+        while (hi > 0) {
+            long long lo = n_com - buf.seg > 0 ? n_com - buf.seg : 0;  // the ring: steps lo .. n_com - 1
+            int pos = slot == 0 ? buf.seg - 1 : slot - 1;               // record of step hi - 1
+            if (hi < n_com) {
+                const long long c = (hi - 1) / stride;
+                const long long base = c * stride;
+                lo = hi - buf.seg > base ? hi - buf.seg : base;
+                Scal R;
+                R.phi0 = S.phi0;
+                double rx, rv, ra1, rc1;
+                ckpt_read(ckw + c * CK_DOUBLES, tl.comp, rx, rv, ra1, rc1, R);
+                long long k = base;
+                while (k < hi) {
+                    const double x0 = rx, v0 = rv, c10 = rc1;
+                    uint32_t rst;
+                    PrimStep RE;
+                    const int r = prim_attempt(P, tl, gs, wi, lane, R, rx, rv, ra1, rc1, RE, rst);
+                    if (r == PA_REJ) continue;
+                    if (r != PA_COMMIT) {
+                        bad = true;
+                        break;
+                    }
+                    if (k >= lo) step_record(srw + (k - lo) * SR_DOUBLES, lane, x0, v0, RE.t, RE.h, c10);
+                    ++k;
                 }
-                if (k >= lo) step_record(srw + (k - lo) * SR_DOUBLES, lane, x0, v0, RE.t, RE.h, c10);
-                ++k;
+                __syncwarp();
+                if (bad) break;
+                pos = (int)(hi - lo) - 1;
             }
-            __syncwarp();
-            if (bad) break;
             for (long long kk = hi - 1; kk >= lo; --kk) {
-                const double* rec = srw + (kk - lo) * SR_DOUBLES;
+                const double* rec = srw + (long long)pos * SR_DOUBLES;
+                pos = pos == 0 ? buf.seg - 1 : pos - 1;
                 const double sx = rec[tl.comp], sv = rec[6 + tl.comp];
                 const double st0 = rec[12], sh0 = rec[13], sc1 = rec[14];
-                adj_step(P, tl, lane, sx, sv, st0, sh0, sc1, S.phi0, false, 0.0, kq, ka, coef, lx, lv, gq, sw);
+                adj_step<false>(P, tl, fl, lane, sx, sv, st0, sh0, sc1, S.phi0, 0.0, kq, ka, lx, lv, gq, sw);
                 adj_rescale(tl, lx, lv, gq, scale_e);
             }
             __syncwarp();

@@ -1261,7 +1261,11 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
             if (tout.ftle && lane == 0) tout.ftle[i] = 0.0;
             continue;
         }
-        const SysDev& P = tab[sid];
+        const SysDev& T = tab[sid];
+        SysDev P;  // the fields that a step needs, in registers
+        P.one = T.one; P.nz = T.nz; P.Omega = T.Omega; P.rtol = T.rtol; P.atol_pos = T.atol_pos;
+        P.atol_vel = T.atol_vel; P.t_max = T.t_max; P.h_max = T.h_max; P.max_attempts = T.max_attempts;
+        P.r0sq = T.r0sq; P.kq_per_q = T.kq_per_q;
         double x, v;
         if (tl.dir == 0) {
             x = __ldg(ic.y0 + yi * ic.ld + i);
@@ -1295,7 +1299,7 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
                 fin.t = 0.0;
                 fin.s_exit = -1.0;
                 fin.status = ST_BAD_IC;
-                store_result(P, ic, out, i, tally(S), fin, false);
+                store_result(T, ic, out, i, tally(S), fin, false);
             }
             if (lane < tin.ndir) {
                 const long long o = (long long)lane * tout.ld + i;
@@ -1305,15 +1309,17 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
             continue;
         }
         // per-lane constants
-        const double kq = tl.comp < 3 ? P.kq[tl.comp] : 0.0;
-        const double ka = tl.comp < 3 ? P.ka[tl.comp] : 0.0;
-        const double coef = tl.comp < 3 ? P.neg_inv_mi : P.inv_ma;
-        double dq_lane = (tl.dir > 0 && used && tl.comp < 3) ? tin.dq[dsel][tl.comp] : 0.0;
-        double dkq = P.kq_per_q * dq_lane;
+        const int axis = tl.comp < 3 ? tl.comp : tl.comp - 3;
+        const double ka = tl.comp < 3 ? T.ka[axis] : P.nz;
+        const double coef = tl.comp < 3 ? T.neg_inv_mi : T.inv_ma;
+        const ForceLane fl = force_lane(T, lane - tl.base);
+        const double dq_axis = (tl.dir > 0 && used) ? tin.dq[dsel][axis] : 0.0;
+        double dq_lane = tl.comp < 3 ? dq_axis : 0.0;
+        double kdq = tl.comp < 3 ? T.kq[axis] : P.kq_per_q * dq_axis;  // see tan_accel
         int scale_e = 0;
         // initial acceleration (FSAL) of primal and tangents, and the initial step of ode45
         double r2, d3[3];
-        double a1 = tan_accel(P, tl, x, cos(S.phi0), kq, ka, dkq, coef, r2, d3);
+        double a1 = tan_accel(P, tl, fl, x, cos(S.phi0), kdq, ka, coef, r2, d3);
         {
             Lane L0;
             for (int k = 0; k < 3; ++k) {
@@ -1321,7 +1327,7 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
                 L0.a1i[k] = shfl(a1, k);
                 L0.a1a[k] = shfl(a1, 3 + k);
             }
-            S.h = initial_step(P, L0);
+            S.h = initial_step(T, L0);
         }
         S.rdot_prev = fma(dd0, vs[3] - vs[0], fma(dd1, vs[4] - vs[1], dd2 * (vs[5] - vs[2])));
         S.t = 0.0; S.hmin = 0.0; S.t_first = 0.0; S.t_last = 0.0;
@@ -1329,7 +1335,7 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
         // |Y0| of direction 1 in the FTLE norm
         double ynorm0 = 0.0;
         {
-            const double sx = x * P.inv_len, sv = v * P.inv_vel;
+            const double sx = x * T.inv_len, sv = v * T.inv_vel;
             double part = fma(sx, sx, sv * sv);
             double acc = 0.0;
 #pragma unroll
@@ -1365,13 +1371,13 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
             const double chsel = lane < 4 ? cv0 : h;
             const double cl = cos(fma(P.Omega, dadd(P, t, chsel), S.phi0));
             const double cs2 = shfl(cl, 0), cs3 = shfl(cl, 1), cs4 = shfl(cl, 2), cs5 = shfl(cl, 3), cs67 = shfl(cl, 4);
-            const double a2 = tan_accel(P, tl, pos2(K, x, v), cs2, kq, ka, dkq, coef, r2, d3);
-            a3 = tan_accel(P, tl, pos3(K, x, v, a1), cs3, kq, ka, dkq, coef, r2, d3);
-            a4 = tan_accel(P, tl, pos4(K, x, v, a1, a2), cs4, kq, ka, dkq, coef, r2, d3);
-            a5 = tan_accel(P, tl, pos5(K, x, v, a1, a2, a3), cs5, kq, ka, dkq, coef, r2, d3);
-            a6 = tan_accel(P, tl, pos6(K, h, x, v, a1, a2, a3, a4), cs67, kq, ka, dkq, coef, r2, d3);
+            const double a2 = tan_accel(P, tl, fl, pos2(K, x, v), cs2, kdq, ka, coef, r2, d3);
+            a3 = tan_accel(P, tl, fl, pos3(K, x, v, a1), cs3, kdq, ka, coef, r2, d3);
+            a4 = tan_accel(P, tl, fl, pos4(K, x, v, a1, a2), cs4, kdq, ka, coef, r2, d3);
+            a5 = tan_accel(P, tl, fl, pos5(K, x, v, a1, a2, a3), cs5, kdq, ka, coef, r2, d3);
+            a6 = tan_accel(P, tl, fl, pos6(K, h, x, v, a1, a2, a3, a4), cs67, kdq, ka, coef, r2, d3);
             xn = pos7(K, h, x, v, a1, a3, a4, a5);
-            a7 = tan_accel(P, tl, xn, cs67, kq, ka, dkq, coef, r2new, dn);
+            a7 = tan_accel(P, tl, fl, xn, cs67, kdq, ka, coef, r2new, dn);
             vn = vel_new(K, v, a1, a3, a4, a5, a6);
             // error test on the primal lanes
             bool okx, fx, okv, fv;
@@ -1415,7 +1421,8 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
             if (tl.dir > 0 && (me > 1023 + 256 || (me > 0 && me < 1023 - 256))) {
                 const int sh = me > 1023 + 256 ? -256 : 256;
                 const double f = sh < 0 ? 0x1p-256 : 0x1p+256;
-                x *= f; v *= f; a1 *= f; dq_lane *= f; dkq *= f;
+                x *= f; v *= f; a1 *= f; dq_lane *= f;
+                if (tl.comp >= 3) kdq *= f;
                 scale_e -= sh;
             }
         }
@@ -1445,7 +1452,7 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
             }
             D.h = h;
             D.t = t;
-            if (lane == 0) finish_exit(P, D, r2new, fin);
+            if (lane == 0) finish_exit(T, D, r2new, fin);
             fin.t = __shfl_sync(FULL, fin.t, 0);
             fin.s_exit = __shfl_sync(FULL, fin.s_exit, 0);
             fin.status = __shfl_sync(FULL, fin.status, 0);
@@ -1514,7 +1521,7 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
             dyf[pi] = shfl(yfx, tl.base + k);
             dyf[pi + 3] = shfl(yfv, tl.base + k);
         }
-        if (lane == 0) store_result(P, ic, out, i, tally(S), fin, true);
+        if (lane == 0) store_result(T, ic, out, i, tally(S), fin, true);
         if (tl.dir > 0 && used && tl.comp == 0) {
             double y0v[12], dy0v[12], dqv[3];
             const double sc = ldexp(1.0, -scale_e);
@@ -1524,7 +1531,7 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
             }
             for (int c = 0; c < 3; ++c) dqv[c] = sc * tin.dq[dsel][c];
             double dth, ddp, dde;
-            obs_derivs(P, S.phi0, y0v, yf, fin.t, dy0v, dyf, dtf_lane, dqv, dth, ddp, dde);
+            obs_derivs(T, S.phi0, y0v, yf, fin.t, dy0v, dyf, dtf_lane, dqv, dth, ddp, dde);
             const long long o = (long long)dsel * tout.ld + i;
             tout.d_theta[o] = ldexp(dth, scale_e);
             tout.d_dp[o] = ldexp(ddp, scale_e);
@@ -1536,7 +1543,7 @@ __global__ void __launch_bounds__(128) k_tangent(const SysDev* __restrict__ tab,
                 double acc = 0.0;
                 for (int c = 0; c < 12; ++c) {
                     const bool vel = (c % 6) >= 3;
-                    const double z = dyf[c] * (vel ? P.inv_vel : P.inv_len);
+                    const double z = dyf[c] * (vel ? T.inv_vel : T.inv_len);
                     acc = fma(z, z, acc);
                 }
                 const double lf = 0.5 * log(acc) + (double)scale_e * 0.69314718055994531;

@@ -107,6 +107,7 @@ constexpr int MAX_TAIL_WARPS = 8;
 // A warp's last trajectory goes on in warp mode: 5.8 us per attempt, 7.7 in group mode, about 20 in lane mode.
 constexpr int LOCAL_MAX = 15;
 constexpr int LOCAL_QUANTUM = 16;
+constexpr int HARD_HOLD = 64;  // attempts of a warp without integer products after one that could not use them
 constexpr int WARP_HOLD = 64;  // attempts in warp mode between looks for records
 // Reserved tail SMs serve trajectories past the slice budget while the bulk still runs. Below this many
 // trajectories per lane the bulk is over before one can get there (131,072 attempts, over 5 s), and the
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(128) k_plain(const SysDev* __restrict__ tab, i
         store_result(P, ic, out, i, tally(L.s), fin, false);
         return;
     }
-    while (lane_attempt(P, L, fin) == RUNNING) {
+    while (lane_attempt<false>(P, L, fin) == RUNNING) {
     }
     store_result(P, ic, out, i, tally(L.s), fin, true);
 }
@@ -173,6 +174,7 @@ __device__ __forceinline__ int lane_phase(const SysDev* __restrict__ tab, int n_
     Final fin;
     long long my = -1;     // trajectory index held by this lane, -1 = idle
     int sid = 0;
+    int hard = 0;          // attempts left with every product on the FP64 unit (warp-uniform)
     bool can_suspend = false;
     bool drained = false;  // the queue has been seen empty by this warp
     const bool may_carry = !part.last;
@@ -240,9 +242,16 @@ __device__ __forceinline__ int lane_phase(const SysDev* __restrict__ tab, int n_
             if (drained) break;
             continue;
         }
+        bool redo = false;
         if (my >= 0) {
             const SysDev& P = tab[sid];
-            if (lane_attempt(P, L, fin) == FINISHED) {
+            int res = REDO;
+            if (hard == 0) res = lane_attempt<true>(P, L, fin);
+            if (res == REDO) {
+                res = lane_attempt<false>(P, L, fin);
+                redo = true;
+            }
+            if (res == FINISHED) {
                 store_result(P, ic, out, my, tally(L.s), fin, true);
                 my = -1;
             } else if (can_suspend && !L.s.retry && L.s.n_acc + L.s.n_rej >= budget) {
@@ -257,6 +266,10 @@ __device__ __forceinline__ int lane_phase(const SysDev* __restrict__ tab, int n_
                 }
             }
         }
+        // a lane that met operands the integer products cannot take: the whole warp goes without for a while
+        // (lanes on both paths would cost both)
+        if (hard > 0) --hard;
+        else if (__any_sync(FULL, redo)) hard = HARD_HOLD;
     }
     return 0;
 }
@@ -1190,26 +1203,19 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
         __threadfence();
         if (atomicAdd(&ctr->warps_done, 1ull) + 1ull == total_warps) atomicMax(&ctr->t_lane_end, global_ns());
     }
-    if (part.lane_only) {
-        // timing runs of the lane phase: trajectories past the budget stay in their suspend records
-    } else if (!part.last) {
-        // only the reserved-SM workers stay: they work on the tail (and lend a hand to the lane phase)
-        // until every lane-phase warp has left, then leave their trajectories for the next part
-        if (r == 1 && budget > 0)
-            while (tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, wait_ok != 0, total_warps, part, n_tc, n_virt,
-                                 true) == 1)
-                lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget, true,
-                           nullptr, 32);
-    } else if (G == 6 && r == 1 && pair && wait_ok) {
+    if (G == 6 && r == 1 && pair && wait_ok && part.last && !part.lane_only) {
         // dedicated tail block: warps 2p and 2p+1 form pair p (chain and helper warp)
         const int w = threadIdx.x >> 5;
         tail_phase_pair(tab, ic, out, susp, ready, ctr, cap, total_warps, &pair_sh[G == 6 ? (w >> 1) : 0],
                         (w & 1) != 0);
-    } else if (r != 2 && budget > 0) {
-        // a reserved-SM worker that finds the tail queue empty runs batches of the lane phase meanwhile
-        const long long help_n = r == 1 ? n_virt : 0;
-        while (tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, wait_ok != 0, total_warps, part, n_tc, help_n, false,
-                             loc, n_loc) == 1)
+    } else if (budget > 0 && !part.lane_only && (part.last ? r != 2 : r == 1)) {
+        // In the last part every warp but a reserved SM's surplus joins the tail. In a part that is not the last
+        // only the reserved SMs' workers stay, until every lane-phase warp has left, and then leave their
+        // trajectories for the next part. A reserved SM's worker that finds the tail queue empty runs batches of
+        // the lane phase meanwhile. (The lane-only timing runs of the autotuner leave trajectories past the
+        // budget in their records.)
+        while (tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, wait_ok != 0, total_warps, part, n_tc,
+                             r == 1 ? n_virt : 0, !part.last, loc, n_loc) == 1)
             n_loc = lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget, true,
                                loc, 32);
     }

@@ -205,6 +205,44 @@ __device__ __forceinline__ double rcp_nr(double x, double one = 1.0)
     return fma(y, fma(r, r, r), y);
 }
 
+// a b to the bit on the integer pipes: the 106-bit product of the mantissas from four 32-bit multiply-adds,
+// rounded to nearest, ties to even. Operands' exponents within 2^+-500 (so that the product is a normal number);
+// otherwise `bad` is set and the value is meaningless (a zero counts as such). About 47 cycles of the integer
+// pipes, which run beside the FP64 unit (a DFMA and this product together take 64); a product on that unit
+// takes 64 of its own.
+__device__ __forceinline__ double soft_mul(double a, double b, bool& bad)
+{
+    const unsigned ah = (unsigned)__double2hiint(a), al = (unsigned)__double2loint(a);
+    const unsigned bh = (unsigned)__double2hiint(b), bl = (unsigned)__double2loint(b);
+    const unsigned ta = (ah & 0xfffffu) | 0x100000u, tb = (bh & 0xfffffu) | 0x100000u;
+    const unsigned long long p = (unsigned long long)al * bl;
+    unsigned long long m = (unsigned long long)al * tb + (p >> 32);
+    m = (unsigned long long)ta * bl + m;
+    const unsigned long long q = (unsigned long long)ta * tb + (m >> 32);  // bits 64.. of the product
+    const unsigned ml = (unsigned)m, ql = (unsigned)q, qh = (unsigned)(q >> 32);
+    const unsigned c = qh >> 9;                                            // 1: the product has 106 bits
+    const unsigned sh = 20u + c;
+    const unsigned rl = __funnelshift_r(ml, ql, sh), rh = __funnelshift_r(ql, qh, sh);
+    const unsigned rem = (ml << (32u - sh)) | min((unsigned)p, 1u);        // below the 53rd bit, and a sticky bit
+    const unsigned long long t = (unsigned long long)rem + (0x7fffffffu + (rl & 1u));
+    const unsigned long long r = (((unsigned long long)rh << 32) | rl) + (t >> 32);
+    unsigned hi = (unsigned)(r >> 32) + (ah & 0x7ff00000u) + (bh & 0x7ff00000u) + (c << 20) - (1024u << 20);
+    hi |= (ah ^ bh) & 0x80000000u;
+    bad = bad || ((ah << 1) - (523u << 21)) > (1000u << 21) || ((bh << 1) - (523u << 21)) > (1000u << 21);
+    return __hiloint2double((int)hi, (int)(unsigned)r);
+}
+
+// A product of the lane-mode step: on the integer pipes (SOFT) or the FP64 unit, the same bits. The lane-mode
+// step is bound by the FP64 unit (586 instructions per attempt) with the integer pipes 15 % busy; 119 of its
+// products go there: the force's after 1/r^2, the step coefficients, the first terms and the tolerances of the
+// error test. 262,144 short trajectories 239.4 -> 216.8 ms, 38,912 at 1.5 uK 78.9 -> 67.6 ms (two warps per
+// sub-partition); a warp alone on its sub-partition, bound by latency, 44.8 -> 46.9 ms.
+template <bool SOFT>
+__device__ __forceinline__ double lmul(const SysDev& P, double a, double b, bool& bad)
+{
+    return SOFT ? soft_mul(a, b, bad) : dmul(P, a, b);
+}
+
 __device__ __forceinline__ double ion_energy(const SysDev& P, double cs, const double xi[3], const double vi[3])
 {
     double k = 0.5 * P.m_i * fma(vi[0], vi[0], fma(vi[1], vi[1], vi[2] * vi[2]));
@@ -216,23 +254,24 @@ __device__ __forceinline__ double ion_energy(const SysDev& P, double cs, const d
 
 // Lane-mode accelerations at positions (xi, xa) with cs = cos(Omega t + phi0) (Eq. 1 and V).
 // Ion: (ka + kq cs) x_i - (g / m_i) d;  atom: (g / m_a) d;  d = x_a - x_i.
+template <bool SOFT>
 __device__ __forceinline__ void accel(const SysDev& P, const double xi[3], const double xa[3], double cs,
-                                      double ai[3], double aa[3], double& r2out, double dout[3])
+                                      double ai[3], double aa[3], double& r2out, double dout[3], bool& bad)
 {
     double d0 = dsub(P, xa[0], xi[0]), d1 = dsub(P, xa[1], xi[1]), d2 = dsub(P, xa[2], xi[2]);
     double r2 = fma(d0, d0, fma(d1, d1, dmul(P, d2, d2)));
     // -V'(r)/(r m) = s^3 (8 C8 s^2 - 4 C4) / m with s = 1/r^2, the 1/m folded into the constants
     const double s = rcp_nr(r2, P.one);
-    const double s2 = dmul(P, s, s);
-    const double s3 = dmul(P, s2, s);
-    const double gmi = dmul(P, s3, fma(P.ci8, s2, -P.ci4));
-    const double gma = dmul(P, s3, fma(P.ca8, s2, -P.ca4));
-    aa[0] = dmul(P, gma, d0);
-    aa[1] = dmul(P, gma, d1);
-    aa[2] = dmul(P, gma, d2);
-    ai[0] = fma(fma(P.kq[0], cs, P.ka[0]), xi[0], dmul(P, gmi, d0));
-    ai[1] = fma(fma(P.kq[1], cs, P.ka[1]), xi[1], dmul(P, gmi, d1));
-    ai[2] = fma(fma(P.kq[2], cs, P.ka[2]), xi[2], dmul(P, gmi, d2));
+    const double s2 = lmul<SOFT>(P, s, s, bad);
+    const double s3 = lmul<SOFT>(P, s2, s, bad);
+    const double gmi = lmul<SOFT>(P, s3, fma(P.ci8, s2, -P.ci4), bad);
+    const double gma = lmul<SOFT>(P, s3, fma(P.ca8, s2, -P.ca4), bad);
+    aa[0] = lmul<SOFT>(P, gma, d0, bad);
+    aa[1] = lmul<SOFT>(P, gma, d1, bad);
+    aa[2] = lmul<SOFT>(P, gma, d2, bad);
+    ai[0] = fma(fma(P.kq[0], cs, P.ka[0]), xi[0], lmul<SOFT>(P, gmi, d0, bad));
+    ai[1] = fma(fma(P.kq[1], cs, P.ka[1]), xi[1], lmul<SOFT>(P, gmi, d1, bad));
+    ai[2] = fma(fma(P.kq[2], cs, P.ka[2]), xi[2], lmul<SOFT>(P, gmi, d2, bad));
     r2out = r2;
     dout[0] = d0;
     dout[1] = d1;
@@ -278,13 +317,25 @@ __device__ __forceinline__ void coef_sh_fill()
     __syncthreads();
 }
 
-__device__ __forceinline__ void coef_all(const SysDev& P, double h, Coef& K)
+template <bool SOFT>
+__device__ __forceinline__ void coef_all(const SysDev& P, double h, Coef& K, bool& bad)
 {
-    K.h2 = dmul(P, h, h);
+    constexpr double TAB[N_COEF] = {
+        DP_C2, DP_C3, DP_C4, DP_C5,
+        DP_AA31, DP_AA41, DP_AA42, DP_AA51, DP_AA52, DP_AA53, DP_AA61, DP_AA62, DP_AA63, DP_AA64,
+        DP_AA71, DP_AA73, DP_AA74, DP_AA75,
+        DP_B1, DP_B3, DP_B4, DP_B5, DP_B6,
+        DP_E1, DP_E3, DP_E4, DP_E5, DP_E6, DP_E7,
+        DP_EA1, DP_EA3, DP_EA4, DP_EA5, DP_EA6};
+    constexpr bool H2[N_COEF] = {false, false, false, false, true, true, true, true, true, true, true, true,
+                                 true, true, true, true, true, true, false, false, false, false, false, false,
+                                 false, false, false, false, false, true, true, true, true, true};
+    K.h2 = lmul<SOFT>(P, h, h, bad);
     double* out = &K.c2;
     const double* sK = coef_sh();
 #pragma unroll
-    for (int k = 0; k < N_COEF; ++k) out[k] = dmul(P, sK[k], COEF_H2[k] ? K.h2 : h);
+    for (int k = 0; k < N_COEF; ++k)
+        out[k] = SOFT ? soft_mul(TAB[k], H2[k] ? K.h2 : h, bad) : dmul(P, sK[k], H2[k] ? K.h2 : h);
 }
 
 __device__ __forceinline__ double pos2(const Coef& K, double x, double v) { return fma(K.c2, v, x); }
@@ -332,6 +383,32 @@ __device__ __forceinline__ void err_check(const SysDev& P, double rtol, double a
 {
     double w = nn_max(dabs(y_old), dabs(y_new));
     sc = nn_max(dmul(P, rtol, w), atol);
+    ae = dabs(e);
+    ok = nn_le(ae, sc);
+    finite = is_finite(y_new) && is_finite(e);
+    ratio = nn_to_float(ae) * __frcp_rn(nn_to_float(sc));
+}
+
+// The same with the first product of a sum, and rtol times the size, as lmul.
+template <bool SOFT>
+__device__ __forceinline__ double err_v(const SysDev& P, bool& bad, const Coef& K, double a1, double a3, double a4,
+                                        double a5, double a6, double a7)
+{
+    return fma(K.e7, a7, fma(K.e6, a6, fma(K.e5, a5, fma(K.e4, a4, fma(K.e3, a3, lmul<SOFT>(P, K.e1, a1, bad))))));
+}
+template <bool SOFT>
+__device__ __forceinline__ double err_x(const SysDev& P, bool& bad, const Coef& K, double a1, double a3, double a4,
+                                        double a5, double a6)
+{
+    return fma(K.f6, a6, fma(K.f5, a5, fma(K.f4, a4, fma(K.f3, a3, lmul<SOFT>(P, K.f1, a1, bad)))));
+}
+template <bool SOFT>
+__device__ __forceinline__ void err_check(const SysDev& P, bool& bad, double rtol, double atol, double y_old,
+                                          double y_new, double e, bool& ok, bool& finite, float& ratio, double& ae,
+                                          double& sc)
+{
+    const double w = nn_max(dabs(y_old), dabs(y_new));
+    sc = nn_max(lmul<SOFT>(P, rtol, w, bad), atol);
     ae = dabs(e);
     ok = nn_le(ae, sc);
     finite = is_finite(y_new) && is_finite(e);
@@ -413,7 +490,7 @@ struct Lane {
     Scal s;
 };
 
-enum LaneResult : int { RUNNING = 0, FINISHED = 1 };
+enum LaneResult : int { RUNNING = 0, FINISHED = 1, REDO = 2 };
 
 // Final state handed to the epilogue.
 struct Final {
@@ -479,7 +556,8 @@ __device__ __forceinline__ bool lane_init(const SysDev& P, const IcPtrs& ic, lon
         return false;
     }
     double r2dummy, dd[3];
-    accel(P, L.xi, L.xa, cos(L.s.phi0), L.a1i, L.a1a, r2dummy, dd);
+    bool bad = false;
+    accel<false>(P, L.xi, L.xa, cos(L.s.phi0), L.a1i, L.a1a, r2dummy, dd, bad);
     L.s.rdot_prev = fma(d0, L.va[0] - L.vi[0], fma(d1, L.va[1] - L.vi[1], d2 * (L.va[2] - L.vi[2])));
     L.s.t = 0.0;
     L.s.h = initial_step(P, L);
@@ -675,8 +753,12 @@ __device__ __noinline__ void finish_exit(const SysDev& P, const StepData& D, dou
 // ---------------------------------------------------------------------------------------------
 // Lane mode: one attempted step. Returns FINISHED when the trajectory is over (fin filled).
 
+// SOFT: part of the products on the integer pipes; REDO when an operand was not an ordinary number (nothing
+// has changed then but what the start of an attempt sets anew).
+template <bool SOFT>
 __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin)
 {
+    bool bad = false;
     uint32_t st = attempt_begin(P, L.s);
     if (st != 0xffffffffu) {
         fin.status = st;
@@ -685,7 +767,7 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
     {
         const double h = L.s.h, t = L.s.t;
         Coef K;
-        coef_all(P, h, K);
+        coef_all<SOFT>(P, h, K, bad);
         double a2i[3], a2a[3], a3i[3], a3a[3], a4i[3], a4a[3], a5i[3], a5a[3], a6i[3], a6a[3], a7i[3], a7a[3];
         double pi_[3], pa_[3], dd[3];
         double r2;
@@ -693,7 +775,7 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
             const double cs = cos(fma(P.Omega, dadd(P, t, K.c2), L.s.phi0));
 #pragma unroll
             for (int j = 0; j < 3; ++j) { pi_[j] = pos2(K, L.xi[j], L.vi[j]); pa_[j] = pos2(K, L.xa[j], L.va[j]); }
-            accel(P, pi_, pa_, cs, a2i, a2a, r2, dd);
+            accel<SOFT>(P, pi_, pa_, cs, a2i, a2a, r2, dd, bad);
         }
         {
             const double cs = cos(fma(P.Omega, dadd(P, t, K.c3), L.s.phi0));
@@ -702,7 +784,7 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
                 pi_[j] = pos3(K, L.xi[j], L.vi[j], L.a1i[j]);
                 pa_[j] = pos3(K, L.xa[j], L.va[j], L.a1a[j]);
             }
-            accel(P, pi_, pa_, cs, a3i, a3a, r2, dd);
+            accel<SOFT>(P, pi_, pa_, cs, a3i, a3a, r2, dd, bad);
         }
         {
             const double cs = cos(fma(P.Omega, dadd(P, t, K.c4), L.s.phi0));
@@ -711,7 +793,7 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
                 pi_[j] = pos4(K, L.xi[j], L.vi[j], L.a1i[j], a2i[j]);
                 pa_[j] = pos4(K, L.xa[j], L.va[j], L.a1a[j], a2a[j]);
             }
-            accel(P, pi_, pa_, cs, a4i, a4a, r2, dd);
+            accel<SOFT>(P, pi_, pa_, cs, a4i, a4a, r2, dd, bad);
         }
         {
             const double cs = cos(fma(P.Omega, dadd(P, t, K.c5), L.s.phi0));
@@ -720,7 +802,7 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
                 pi_[j] = pos5(K, L.xi[j], L.vi[j], L.a1i[j], a2i[j], a3i[j]);
                 pa_[j] = pos5(K, L.xa[j], L.va[j], L.a1a[j], a2a[j], a3a[j]);
             }
-            accel(P, pi_, pa_, cs, a5i, a5a, r2, dd);
+            accel<SOFT>(P, pi_, pa_, cs, a5i, a5a, r2, dd, bad);
         }
         const double cs_end = cos(fma(P.Omega, dadd(P, t, h), L.s.phi0));  // stages 6 and 7 share t + h
         {
@@ -729,7 +811,7 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
                 pi_[j] = pos6(K, h, L.xi[j], L.vi[j], L.a1i[j], a2i[j], a3i[j], a4i[j]);
                 pa_[j] = pos6(K, h, L.xa[j], L.va[j], L.a1a[j], a2a[j], a3a[j], a4a[j]);
             }
-            accel(P, pi_, pa_, cs_end, a6i, a6a, r2, dd);
+            accel<SOFT>(P, pi_, pa_, cs_end, a6i, a6a, r2, dd, bad);
         }
         double xni[3], xna[3], vni[3], vna[3];
         double r2new;
@@ -738,7 +820,7 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
             xni[j] = pos7(K, h, L.xi[j], L.vi[j], L.a1i[j], a3i[j], a4i[j], a5i[j]);
             xna[j] = pos7(K, h, L.xa[j], L.va[j], L.a1a[j], a3a[j], a4a[j], a5a[j]);
         }
-        accel(P, xni, xna, cs_end, a7i, a7a, r2new, dd);  // dd = x_a,new - x_i,new
+        accel<SOFT>(P, xni, xna, cs_end, a7i, a7a, r2new, dd, bad);  // dd = x_a,new - x_i,new
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             vni[j] = vel_new(K, L.vi[j], L.a1i[j], a3i[j], a4i[j], a5i[j], a6i[j]);
@@ -755,15 +837,16 @@ __device__ __forceinline__ int lane_attempt(const SysDev& P, Lane& L, Final& fin
             bool ok, fi;
             float r;
             double ae, sc;
-            err_check(P, P.rtol, P.atol_pos, L.xi[j], xni[j], err_x(P, K, L.a1i[j], a3i[j], a4i[j], a5i[j], a6i[j]), ok, fi, r, ae, sc);
+            err_check<SOFT>(P, bad, P.rtol, P.atol_pos, L.xi[j], xni[j], err_x<SOFT>(P, bad, K, L.a1i[j], a3i[j], a4i[j], a5i[j], a6i[j]), ok, fi, r, ae, sc);
             accept = accept && ok; finite = finite && fi; err_take(em, r, 2 * j, ae, sc);
-            err_check(P, P.rtol, P.atol_vel, L.vi[j], vni[j], err_v(P, K, L.a1i[j], a3i[j], a4i[j], a5i[j], a6i[j], a7i[j]), ok, fi, r, ae, sc);
+            err_check<SOFT>(P, bad, P.rtol, P.atol_vel, L.vi[j], vni[j], err_v<SOFT>(P, bad, K, L.a1i[j], a3i[j], a4i[j], a5i[j], a6i[j], a7i[j]), ok, fi, r, ae, sc);
             accept = accept && ok; finite = finite && fi; err_take(em, r, 2 * j + 1, ae, sc);
-            err_check(P, P.rtol, P.atol_pos, L.xa[j], xna[j], err_x(P, K, L.a1a[j], a3a[j], a4a[j], a5a[j], a6a[j]), ok, fi, r, ae, sc);
+            err_check<SOFT>(P, bad, P.rtol, P.atol_pos, L.xa[j], xna[j], err_x<SOFT>(P, bad, K, L.a1a[j], a3a[j], a4a[j], a5a[j], a6a[j]), ok, fi, r, ae, sc);
             accept = accept && ok; finite = finite && fi; err_take(em, r, 2 * (3 + j), ae, sc);
-            err_check(P, P.rtol, P.atol_vel, L.va[j], vna[j], err_v(P, K, L.a1a[j], a3a[j], a4a[j], a5a[j], a6a[j], a7a[j]), ok, fi, r, ae, sc);
+            err_check<SOFT>(P, bad, P.rtol, P.atol_vel, L.va[j], vna[j], err_v<SOFT>(P, bad, K, L.a1a[j], a3a[j], a4a[j], a5a[j], a6a[j], a7a[j]), ok, fi, r, ae, sc);
             accept = accept && ok; finite = finite && fi; err_take(em, r, 2 * (3 + j) + 1, ae, sc);
         }
+        if (SOFT && bad) return REDO;
         if (!finite) {
             fin.status = ST_NONFINITE;
             goto stop_here;

@@ -19,7 +19,7 @@
 // sub-partition 64-76 cycles on this GPU, so adding the 32 values of a row one after the other (64 FP64
 // instructions per row) took 470 us of 659 us, and the global atomics of every trajectory most of the
 // rest; lane-wise sums take two FP64 instructions per row, and one atomic per count and cell change:
-// 108 us (2^22 trajectories in 250 cells laid out cell by cell).
+// 108 us (2^22 trajectories in 250 cells laid out cell by cell), 86.5 us with the rows loaded ahead.
 #pragma once
 
 #include <cstdint>
@@ -108,7 +108,44 @@ __device__ __forceinline__ void flush_run(CellRun& r, int c, int lane, ia_stats*
     r.s1 = r.s2 = 0.0;
 }
 
-// chunk: trajectories per warp, a multiple of 32.
+// One lane's trajectory of a row.
+struct StatsRow {
+    int c, nb;
+    uint32_t status;
+    int steps, rej;
+    double dE;
+    double t0, t1;  // first and last bounce of a complex
+};
+__device__ __forceinline__ StatsRow load_row(const ObsPtrs& obs, const int32_t* __restrict__ cell, long long i,
+                                             long long hi, int n_cells)
+{
+    StatsRow r;
+    r.c = -1;
+    r.nb = r.steps = r.rej = 0;
+    r.status = 0u;
+    r.dE = r.t0 = r.t1 = 0.0;
+    if (i < hi) {
+        r.c = cell ? __ldg(cell + i) : 0;
+        if (r.c < 0 || r.c >= n_cells) r.c = -1;
+        r.status = obs.status[i];
+        r.nb = obs.n_bounce[i];
+        r.steps = obs.n_steps[i];
+        r.rej = obs.n_rej[i];
+        r.dE = obs.dE_ion[i];
+    }
+    return r;
+}
+
+__device__ __forceinline__ void load_bounces(const ObsPtrs& obs, long long i, StatsRow& r)
+{
+    if (r.c >= 0 && r.nb >= 2) {
+        r.t0 = obs.t_first[i];
+        r.t1 = obs.t_last[i];
+    }
+}
+
+// chunk: trajectories per warp, a multiple of 32. A warp's rows follow one another: two are loaded ahead of
+// the one that is counted, and the bounce times of the next one's complexes.
 __global__ void __launch_bounds__(STATS_BLOCK) k_stats_pass1(ObsPtrs obs, long long n, const int32_t* __restrict__ cell,
                                                              int n_cells, ia_stats* __restrict__ st,
                                                              double* __restrict__ partial, long long chunk)
@@ -129,24 +166,20 @@ __global__ void __launch_bounds__(STATS_BLOCK) k_stats_pass1(ObsPtrs obs, long l
     r.att = 0ull;
     r.s1 = r.s2 = 0.0;
     int cur = -1;  // cell of the run held in registers
-#pragma unroll 2
+    StatsRow n1 = load_row(obs, cell, lo + lane, hi, n_cells), n2 = load_row(obs, cell, lo + 32 + lane, hi, n_cells);
+    load_bounces(obs, lo + lane, n1);
     for (long long base = lo; base < hi; base += 32) {
         const long long i = base + lane;
-        const bool in = i < hi;
-        int c = -1, nb = 0;
-        uint32_t status = 0;
-        long long att = 0;
-        double dE = 0.0;
-        if (in) {
-            c = cell ? __ldg(cell + i) : 0;
-            if (c < 0 || c >= n_cells) c = -1;
-            status = obs.status[i];
-            nb = obs.n_bounce[i];
-            att = (long long)obs.n_steps[i] + (long long)obs.n_rej[i];
-            dE = obs.dE_ion[i];
-        }
+        const StatsRow row = n1;
+        n1 = n2;
+        load_bounces(obs, i + 32, n1);
+        n2 = load_row(obs, cell, i + 64, hi, n_cells);
+        const int c = row.c, nb = row.nb;
+        const uint32_t status = row.status;
+        const long long att = (long long)row.steps + (long long)row.rej;
+        const double dE = row.dE;
         const int c0 = __shfl_sync(0xffffffffu, c, 0);
-        const int lt = c >= 0 && nb >= 2 ? lifetime_bin(obs.t_last[i] - obs.t_first[i]) : 0;
+        const int lt = c >= 0 && nb >= 2 ? lifetime_bin(row.t1 - row.t0) : 0;
         if (__all_sync(0xffffffffu, c == c0)) {
             if (c0 < 0) continue;
             if (c0 != cur) {

@@ -173,9 +173,11 @@ int ia_reserve(ia_system* sys, int64_t n, const ia_launch_opts* opts);
  * n = 0 is a no-op. opts may be NULL (defaults).
  * Persistent launches: a trajectory that has used opts->slice_budget attempted steps is saved to a
  * suspend record and finished by tail workers that give each such trajectory a group of lanes, which
- * run its steps ~2.2x faster; tail workers start at once on opts->tail_sms SMs and every other warp
- * joins them once the queue is drained (one cooperative launch, every wait bounded). Results are
- * bit-identical to the plain kernel.
+ * run its steps ~2.6x faster; tail workers start at once on opts->tail_sms SMs and every other warp
+ * joins them once the queue is drained (one cooperative launch, every wait bounded). With slice_budget
+ * 0, small batches and what is left of a large one when its queue is empty move to groups of lanes
+ * before the budget, and SMs are reserved only for batches of at least 8 trajectories per lane of the
+ * grid. Results are bit-identical to the plain kernel.
  * Concurrency: persistent launches that share the system's own scratch must not overlap; pass a
  * distinct opts->scratch to run them concurrently.
  */

@@ -26,9 +26,9 @@
 // This file spends FP64 instructions only on the method's arithmetic:
 //   * stage velocities are never formed (Nystrom form, gen_dp5_nystrom.py);
 //   * comparisons and max/min of non-negative doubles are integer operations on their bit patterns;
-//   * 1/r^2 is a Newton-Raphson refinement of an FP32 seed (two iterations, ~1 ulp);
-//   * the step-size factor (a smooth function of the error ratio, not a decision) is computed in
-//     FP32; the accept/reject decision stays exact in FP64;
+//   * 1/r^2 is one third-order refinement of an FP32 seed (~1 ulp);
+//   * the step-size factor is an FP32 seed refined by one Newton step in FP64; the accept/reject
+//     decision is exact;
 //   * float <-> double conversions are integer operations on the bit patterns;
 //   * in group mode, per-step scalars are spread over the lanes of a group and exchanged by shuffles,
 //     and two independent products share one FMA instruction on different lanes.

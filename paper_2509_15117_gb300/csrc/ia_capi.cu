@@ -105,6 +105,9 @@ constexpr int MAX_TAIL_WARPS = 8;
 // attempts 1,212 -> 321 ms, 50,000 thermal ones of up to 8,192 243 -> 94 ms, the 40-system sweep of 67,240
 // 324 -> 309 ms; 262,144 trajectories of one length, which end together, 239 -> 241 ms.
 // A warp's last trajectory goes on in warp mode: 5.8 us per attempt, 7.7 in group mode, about 20 in lane mode.
+// The line at 15, measured with the integer products in lane mode (ms at 10 / 15 / 20: thermal 93.8 / 88.8 /
+// 85.0, sweep 280 / 275 / 290, the sweep in four parts of up to 32,768 attempts 745 / 645 / 626, mixed graph
+// 350 / 334 / 340, 262,144 of one length 218.5 / 218.5 / 223.6).
 constexpr int LOCAL_MAX = 15;
 constexpr int LOCAL_QUANTUM = 16;
 constexpr int HARD_HOLD = 64;  // attempts of a warp without integer products after one that could not use them

@@ -176,7 +176,8 @@ int ia_reserve(ia_system* sys, int64_t n, const ia_launch_opts* opts);
  * run its steps ~2.6x faster; tail workers start at once on opts->tail_sms SMs and every other warp
  * joins them once the queue is drained (one cooperative launch, every wait bounded). With slice_budget
  * 0, small batches and what is left of a large one when its queue is empty move to groups of lanes
- * before the budget, and SMs are reserved only for batches of at least 8 trajectories per lane of the
+ * before the budget (which holds there too: a warp hands on those past it while it has more than it can
+ * advance at once), and SMs are reserved only for batches of at least 8 trajectories per lane of the
  * grid. Results are bit-identical to the plain kernel.
  * Concurrency: persistent launches that share the system's own scratch must not overlap; pass a
  * distinct opts->scratch to run them concurrently.
@@ -517,6 +518,20 @@ int ia_philox4x64(uint64_t key0, uint64_t key1, uint64_t ctr1, int64_t first, in
  */
 int ia_sample_ics(const ia_sampler* s, int64_t first, int64_t n, double* y0, double* phi0, int64_t ld,
                   void* stream);
+
+/*
+ * Test hook (no counterpart in the paper): launches on `sys` with slice_budget 0 use `budget` attempted
+ * steps instead of 131072 (0: 131072 again), so that short trajectories reach the paths of long ones.
+ * Results do not depend on it. No launch on the system may be under way in another thread.
+ */
+int ia_test_limits(ia_system* sys, int32_t budget);
+
+/*
+ * Test hook (no counterpart in the paper): suspend records taken by the latest persistent launch on the
+ * system's own scratch (q NULL) or by a queue's batch so far (the count runs on when the records are
+ * used up), and the SMs that its latest launch reserved for the tail. Synchronous.
+ */
+int ia_test_tail(const ia_system* sys, const ia_queue* q, int64_t* records, int64_t* reserved);
 
 /*
  * Test hook (no counterpart in the paper): y[i] = 1/x[i] computed as the integrator computes 1/r^2

@@ -34,7 +34,8 @@ EXPORTED = ("ia_system_create", "ia_system_destroy", "ia_system_count", "ia_scra
             "ia_graph_launch", "ia_graph_destroy", "ia_autotune", "ia_launch_phases", "ia_launch_tangent",
             "ia_adjoint_scratch_bytes", "ia_launch_adjoint", "ia_philox4x64", "ia_sample_ics", "ia_fp64_peak",
             "ia_rcp_check", "ia_error_string", "ia_version", "ia_queue_create", "ia_queue_launch",
-            "ia_queue_reset", "ia_queue_state", "ia_queue_phases", "ia_queue_destroy", "ia_static_phases")
+            "ia_queue_reset", "ia_queue_state", "ia_queue_phases", "ia_queue_destroy", "ia_static_phases",
+            "ia_test_limits", "ia_test_tail")
 
 IA_SAMPLE_HEAD_ON = 0
 IA_SAMPLE_SPHERE = 1
@@ -240,6 +241,11 @@ def load(build_if_missing: bool = True):
     L.ia_reserve.restype = ctypes.c_int
     L.ia_rcp_check.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
     L.ia_rcp_check.restype = ctypes.c_int
+    L.ia_test_limits.argtypes = [ctypes.c_void_p, ctypes.c_int32]
+    L.ia_test_limits.restype = ctypes.c_int
+    L.ia_test_tail.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.POINTER(ctypes.c_int64),
+                               ctypes.POINTER(ctypes.c_int64)]
+    L.ia_test_tail.restype = ctypes.c_int
     L.ia_philox4x64.argtypes = [ctypes.c_uint64, ctypes.c_uint64, ctypes.c_uint64, ctypes.c_int64, ctypes.c_int64,
                                 ctypes.c_void_p, ctypes.c_void_p]
     L.ia_philox4x64.restype = ctypes.c_int
@@ -404,6 +410,17 @@ def ia_rcp_check(x, y, stream=None) -> None:
     _tensor(x, "x", torch.float64, (None,))
     _tensor(y, "y", torch.float64, (x.shape[0],))
     _check(load().ia_rcp_check(x.data_ptr(), y.data_ptr(), int(x.numel()), _stream_ptr(stream)))
+
+
+def ia_test_limits(handle: int, budget: int = 0) -> None:
+    _check(load().ia_test_limits(handle, int(budget)))
+
+
+def ia_test_tail(handle: int, queue: "Queue | None" = None) -> tuple:
+    """(suspend records taken, SMs reserved for the tail); see ionatom.h."""
+    a, b = ctypes.c_int64(), ctypes.c_int64()
+    _check(load().ia_test_tail(handle, queue.ptr if queue is not None else None, ctypes.byref(a), ctypes.byref(b)))
+    return a.value, b.value
 
 
 def make_sampler(kind: int, desc: dict, seed: int, E: float = 0.0, kT: float = 0.0, kT_ion: float = 0.0,

@@ -58,6 +58,8 @@ struct Counters {
     unsigned long long tail;        // next suspend record to resume
     unsigned long long carry_n[2];  // lane-mode carry records written into buffer 0 / 1
     unsigned long long tcarry_n[2]; // group-mode carry records written into buffer 0 / 1
+    // --- written by every launch ---
+    unsigned long long reserved;    // SMs whose first block is a tail worker
 };
 constexpr size_t SCRATCH_HEAD = 1024;
 static_assert(sizeof(Counters) <= SCRATCH_HEAD, "scratch head");
@@ -104,6 +106,9 @@ constexpr int MAX_TAIL_WARPS = 8;
 // Against lane mode to the end: one Rb trajectory of 8,192 attempts 128 -> 64 ms, 1,024 of up to 32,768
 // attempts 1,212 -> 321 ms, 50,000 thermal ones of up to 8,192 243 -> 94 ms, the 40-system sweep of 67,240
 // 324 -> 309 ms; 262,144 trajectories of one length, which end together, 239 -> 241 ms.
+// The slice budget holds for them too: while a warp has more than one batch, those past the budget go to
+// suspend records, and idle warps take them (twelve neighbours in the queue of 40,000 trajectories, 10^6 attempts
+// each, which one warp would otherwise carry to their end: 17.6 -> 8.9 s).
 // A warp's last trajectory goes on in warp mode: 5.8 us per attempt, 7.7 in group mode, about 20 in lane mode.
 // The line at 15, measured with the integer products in lane mode (ms at 10 / 15 / 20: thermal 93.8 / 88.8 /
 // 85.0, sweep 280 / 275 / 290, the sweep in four parts of up to 32,768 attempts 745 / 645 / 626, mixed graph
@@ -295,6 +300,41 @@ __device__ __forceinline__ bool claim_record(Counters* ctr, long long cap, unsig
     return false;
 }
 
+// A warp has left the lane phase: it publishes no more records. (A reserved SM's worker counts from the start;
+// what it publishes later it can take itself.)
+__device__ __forceinline__ void leave_lane_phase(Counters* ctr, unsigned long long total_warps)
+{
+    if ((threadIdx.x & 31) == 0) {
+        __threadfence();
+        if (atomicAdd(&ctr->warps_done, 1ull) + 1ull == total_warps) atomicMax(&ctr->t_lane_end, global_ns());
+    }
+}
+
+// Local trajectories past the budget go to suspend records while the warp keeps more than `keep`; returns the
+// mask of those that stay. more: whether others may still pass it (and there was room).
+__device__ __noinline__ unsigned publish_local(const SysDev* __restrict__ tab, const Susp* loc, unsigned alive, int keep,
+                                               int budget, Counters* __restrict__ ctr, unsigned* __restrict__ ready,
+                                               Susp* __restrict__ susp, long long cap, bool& more)
+{
+    const int l = threadIdx.x & 31;
+    const bool mine = (alive >> l) & 1u;
+    const bool over = mine && loc[l].n_acc + loc[l].n_rej >= budget;
+    const int rank = __popc(__ballot_sync(FULL, over) & ((1u << l) - 1u));
+    const bool want = over && rank < __popc(alive) - keep;
+    unsigned long long slot = ~0ull;
+    if (want) slot = atomicAdd(&ctr->n_susp, 1ull);
+    const bool room = slot < (unsigned long long)cap;
+    if (room) {
+        susp[slot] = loc[l];
+        __threadfence();
+        atomicExch(ready + slot, 1u);
+    }
+    const unsigned left = alive & ~__ballot_sync(FULL, room);
+    more = !__any_sync(FULL, want && !room) && __popc(left) > keep &&
+           __any_sync(FULL, mine && !room && tab[loc[l].sid].max_attempts > budget);
+    return left;
+}
+
 // Tail phase (group mode): one suspended trajectory per group of G lanes until it ends.
 // wait_ok: records may still be written by warps in the lane phase (all blocks co-resident,
 // cooperative launch), so an idle group waits for them, boundedly; otherwise an idle group stops
@@ -309,15 +349,16 @@ __device__ __forceinline__ bool claim_record(Counters* ctr, long long cap, unsig
 // The group-mode carry records of the previous part (part.tcarry_in, n_tc of them) are resumed before
 // any suspend record: they hold the trajectories that part's tail was running, the oldest in the tail.
 // A yield writes to part.tcarry_out, or, when that is full, appends a suspend record.
-// loc, n_loc: trajectories the warp brings from the lane phase (records in shared memory, at most
-// LOCAL_MAX). They come before any other record and advance in turns, 32 / G at a time.
+// loc, alive: trajectories the warp brings from the lane phase (records in shared memory, at most
+// LOCAL_MAX; the mask of those that are left). They come before any other record and advance in turns, 32 / G
+// at a time. turns >= 0: after that many turns, or with no more than 32 / G of them left, returns 2 with all of
+// them in their records, so that its caller can publish those past the budget.
 template <int G>
 __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const IcPtrs& ic, const ObsPtrs& out,
                                           Susp* __restrict__ susp, unsigned* __restrict__ ready,
                                           Counters* __restrict__ ctr, long long cap, bool wait_ok,
                                           unsigned long long total_warps, const Part& part, long long n_tc,
-                                          long long help_n = 0, bool may_yield = false, Susp* loc = nullptr,
-                                          int n_loc = 0)
+                                          long long help_n, bool may_yield, Susp* loc, unsigned& alive, int turns)
 {
     constexpr int R = (N_COEF + G - 1) / G;  // coefficient rounds per lane
     constexpr int NG = 32 / G;               // groups per warp
@@ -335,7 +376,7 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
     bool yield_room = true;   // false once a yield found the record area full (warp-uniform)
     // local records: unfinished ones, those not held by a group now, this group's (-1: none), the first of
     // the next turn, attempts left of this turn (all but lslot warp-uniform)
-    unsigned lalive = (1u << n_loc) - 1u, lpend = lalive;
+    unsigned lalive = alive, lpend = lalive;
     int lslot = -1, lnext = 0, lturn = 0;
     // warp mode (G = 6): while the warp has a single trajectory, every group holds a copy of it and group 0
     // answers for it; left every WARP_HOLD attempts to look for records
@@ -376,6 +417,10 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
                     }
                 }
                 __syncwarp();
+                if (turns >= 0 && (turns-- == 0 || __popc(lalive) <= NG)) {
+                    alive = lalive;
+                    return 2;
+                }
                 const int grp = gl.base / G, n_al = __popc(lalive);
                 int first = __popc(lalive & ((1u << lnext) - 1u));  // rank of the first to take
                 if (first >= n_al) first = 0;
@@ -452,7 +497,8 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
             if (!__any_sync(FULL, active)) return 0;
         }
         const bool need = !active && !drained && lpend == 0u;
-        bool poll = __any_sync(FULL, need);
+        const unsigned needy = __ballot_sync(FULL, need && gl.c == 0);
+        bool poll = needy != 0u;
         if (poll && claim_skip > 0 && __any_sync(FULL, active)) {
             // an idle group polls the record counters (global atomics, microseconds) only every
             // CLAIM_BACKOFF attempts while its warp still runs other trajectories
@@ -460,15 +506,18 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
             poll = false;
         }
         if (poll) {
-            // the group's first lane claims; the claim is broadcast to the group
+            // One group claims at a time, so that records published together go to several idle warps (five
+            // in one warp step at 7.7 us per attempt, one at 5.8); its first lane does, for the whole warp.
+            const int asker = __ffs((int)needy) - 1;
+            const bool ask = (int)(threadIdx.x & 31) == asker;
             int got = 0;
             unsigned long long k = 0;
-            if (need && gl.c == 0 && n_tc > 0 &&
+            if (ask && n_tc > 0 &&
                 *(volatile unsigned long long*)&ctr->tc_taken < (unsigned long long)n_tc) {
                 k = atomicAdd(&ctr->tc_taken, 1ull);
                 if (k < (unsigned long long)n_tc) got = 4;  // a trajectory the previous part's tail ran
             }
-            if (need && gl.c == 0 && got == 0) {
+            if (ask && got == 0) {
                 if (claim_record(ctr, cap, k)) {
                     got = 1;
                     unsigned spins = 0;
@@ -501,11 +550,11 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
                     }
                 }
             }
-            got = __shfl_sync(FULL, got, gl.base);
-            k = __shfl_sync(FULL, k, gl.base);
-            if (!__any_sync(FULL, need && (got == 1 || got == 4))) claim_skip = CLAIM_BACKOFF;
+            got = __shfl_sync(FULL, got, asker);
+            k = __shfl_sync(FULL, k, asker);
+            claim_skip = CLAIM_BACKOFF;
             if (need) {
-                if (got == 1 || got == 4) {
+                if ((got == 1 || got == 4) && gl.base == asker) {
                     // written by another SM during this launch (or by the previous launch): read through L2
                     const Susp* r = (got == 4 ? part.tcarry_in : susp) + k;
                     x = __ldcg(&r->x[gl.comp]);
@@ -1179,6 +1228,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
         asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
         if (smid < (unsigned)MAX_TAIL_SMS) rank = atomicAdd(&ctr->sm_claim[smid], 1u);
         role = reserve && smid < (unsigned)tail_sms && smid < (unsigned)MAX_TAIL_SMS ? (rank == 0u ? 1 : 2) : 0;
+        if (blockIdx.x == 0) ctr->reserved = reserve ? (unsigned long long)tail_sms : 0ull;
         sm_rank = (int)rank;
     }
     __syncthreads();
@@ -1202,10 +1252,8 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
     if (r == 0 && share > 0)
         n_loc = lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget, false,
                            loc, share);
-    if ((threadIdx.x & 31) == 0) {
-        __threadfence();
-        if (atomicAdd(&ctr->warps_done, 1ull) + 1ull == total_warps) atomicMax(&ctr->t_lane_end, global_ns());
-    }
+    bool owes = n_loc > 32 / G;  // may publish local trajectories: counts itself later
+    if (!owes) leave_lane_phase(ctr, total_warps);
     if (G == 6 && r == 1 && pair && wait_ok && part.last && !part.lane_only) {
         // dedicated tail block: warps 2p and 2p+1 form pair p (chain and helper warp)
         const int w = threadIdx.x >> 5;
@@ -1217,10 +1265,28 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
         // trajectories for the next part. A reserved SM's worker that finds the tail queue empty runs batches of
         // the lane phase meanwhile. (The lane-only timing runs of the autotuner leave trajectories past the
         // budget in their records.)
-        while (tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, wait_ok != 0, total_warps, part, n_tc,
-                             r == 1 ? n_virt : 0, !part.last, loc, n_loc) == 1)
-            n_loc = lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget, true,
-                               loc, 32);
+        // (The empty asm keeps the two loops apart for the compiler; merged, an attempt took 2 % longer.)
+        unsigned alive = (1u << n_loc) - 1u;
+#pragma unroll 1
+        for (;;) {
+            bool more = false;
+            asm volatile("" : "+r"(alive) : : "memory");
+            if (__popc(alive) > 32 / G)
+                alive = publish_local(tab, loc, alive, 32 / G, budget, ctr, ready, susp, cap, more);
+            // (budget / 1,024 turns of LOCAL_QUANTUM attempts: a look every few ms)
+            if (owes && !more) {
+                leave_lane_phase(ctr, total_warps);
+                owes = false;
+            }
+            const int rc = tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, wait_ok != 0, total_warps, part, n_tc,
+                                         r == 1 ? n_virt : 0, !part.last, loc, alive, more ? (budget >> 10) + 1 : -1);
+            if (rc == 0) break;
+            if (rc == 1) {
+                n_loc = lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget,
+                                   true, loc, 32);
+                alive = (1u << n_loc) - 1u;
+            }
+        }
     }
     if ((threadIdx.x & 31) == 0) atomicMax(&ctr->t_end, global_ns());
 }
@@ -1237,7 +1303,8 @@ __global__ void __launch_bounds__(128) k_tail(const SysDev* __restrict__ tab, Ic
         const unsigned long long c = *part.tcarry_in_n;
         n_tc = c < (unsigned long long)part.tcarry_cap ? (long long)c : part.tcarry_cap;
     }
-    tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, false, 0ull, part, n_tc);
+    unsigned none = 0u;
+    tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, false, 0ull, part, n_tc, 0, false, nullptr, none, -1);
     if ((threadIdx.x & 31) == 0) atomicMax(&ctr->t_end, global_ns());
 }
 
@@ -1596,6 +1663,7 @@ struct ia_system {
     void* d_adj_scratch;      // checkpoints and step buffers of adjoint launches (grown on demand)
     size_t adj_scratch_bytes;
     int num_sms;
+    int default_budget;       // slice budget of launches that leave it to the library
 };
 
 struct ia_graph {
@@ -1842,7 +1910,7 @@ int sched_config(const ia_system* sys, const Resolved& r, SchedCfg& c)
     // Waiting for records across blocks needs every block resident: a cooperative launch gives that.
     int coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, sys->device);
-    c.budget = o.slice_budget > 0 ? o.slice_budget : 0;
+    c.budget = r.default_budget ? sys->default_budget : (o.slice_budget > 0 ? o.slice_budget : 0);
     c.wait_ok = (c.budget > 0 && coop && c.grid <= c.resident * sys->num_sms) ? 1 : 0;
     c.tail_sms = (c.wait_ok && o.tail_sms > 0) ? o.tail_sms : 0;
     if (c.tail_sms > sys->num_sms / 2) c.tail_sms = sys->num_sms / 2;
@@ -1949,6 +2017,7 @@ int ia_system_create(const ia_system_desc* desc, int32_t n_sys, ia_system** out)
     s->d_adj_scratch = nullptr;
     s->adj_scratch_bytes = 0;
     s->num_sms = prop.multiProcessorCount;
+    s->default_budget = DEFAULT_BUDGET;
     if (cudaMalloc(&s->d_tab, sizeof(SysDev) * (size_t)n_sys) != cudaSuccess ||
         cudaMemcpy(s->d_tab, host, sizeof(SysDev) * (size_t)n_sys, cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaFree(s->d_tab);
@@ -2629,6 +2698,25 @@ int ia_launch_phases(ia_system* sys, const void* scratch, double* lane_ms, doubl
     *lane_ms = c.t_lane_end >= c.t_start ? 1e-6 * (double)(c.t_lane_end - c.t_start) : 0.0;
     *total_ms = 1e-6 * (double)(c.t_end - c.t_start);
     if (errors) *errors = (int64_t)c.errors;
+    return IA_OK;
+}
+
+int ia_test_limits(ia_system* sys, int32_t budget)
+{
+    if (!sys || budget < 0) return IA_ERR_INVALID_ARG;
+    sys->default_budget = budget ? budget : DEFAULT_BUDGET;
+    return IA_OK;
+}
+
+int ia_test_tail(const ia_system* sys, const ia_queue* q, int64_t* records, int64_t* reserved)
+{
+    if (!sys || !records || !reserved || (q && q->sys != sys)) return IA_ERR_INVALID_ARG;
+    const void* base = q ? q->scratch : sys->d_scratch;
+    if (!base || (q && q->parts == 0)) return IA_ERR_INVALID_ARG;
+    Counters c;
+    if (cudaMemcpy(&c, base, sizeof(Counters), cudaMemcpyDeviceToHost) != cudaSuccess) return IA_ERR_CUDA;
+    *records = (int64_t)c.n_susp;
+    *reserved = (int64_t)c.reserved;
     return IA_OK;
 }
 

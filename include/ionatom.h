@@ -177,8 +177,9 @@ int ia_reserve(ia_system* sys, int64_t n, const ia_launch_opts* opts);
  * joins them once the queue is drained (one cooperative launch, every wait bounded). With slice_budget
  * 0, small batches and what is left of a large one when its queue is empty move to groups of lanes
  * before the budget (which holds there too: a warp hands on those past it while it has more than it can
- * advance at once), and SMs are reserved only for batches of at least 8 trajectories per lane of the
- * grid. Results are bit-identical to the plain kernel.
+ * advance at once), and with tail_sms 0 too, SMs are reserved only for batches of at least 8
+ * trajectories per lane of the grid (or when the previous part of a queue left trajectories in group
+ * mode). Results are bit-identical to the plain kernel.
  * Concurrency: persistent launches that share the system's own scratch must not overlap; pass a
  * distinct opts->scratch to run them concurrently.
  */
@@ -521,10 +522,11 @@ int ia_sample_ics(const ia_sampler* s, int64_t first, int64_t n, double* y0, dou
 
 /*
  * Test hook (no counterpart in the paper): launches on `sys` with slice_budget 0 use `budget` attempted
- * steps instead of 131072 (0: 131072 again), so that short trajectories reach the paths of long ones.
- * Results do not depend on it. No launch on the system may be under way in another thread.
+ * steps instead of 131072 (0: 131072 again), so that short trajectories reach the paths of long ones,
+ * and with tail_sms 0 they reserve SMs from reserve_rounds trajectories per lane on instead of 8 (-1: 8
+ * again). Results do not depend on either. No launch on the system may be under way in another thread.
  */
-int ia_test_limits(ia_system* sys, int32_t budget);
+int ia_test_limits(ia_system* sys, int32_t budget, int32_t reserve_rounds);
 
 /*
  * Test hook (no counterpart in the paper): suspend records taken by the latest persistent launch on the

@@ -241,7 +241,7 @@ def load(build_if_missing: bool = True):
     L.ia_reserve.restype = ctypes.c_int
     L.ia_rcp_check.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
     L.ia_rcp_check.restype = ctypes.c_int
-    L.ia_test_limits.argtypes = [ctypes.c_void_p, ctypes.c_int32]
+    L.ia_test_limits.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32]
     L.ia_test_limits.restype = ctypes.c_int
     L.ia_test_tail.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.POINTER(ctypes.c_int64),
                                ctypes.POINTER(ctypes.c_int64)]
@@ -412,8 +412,8 @@ def ia_rcp_check(x, y, stream=None) -> None:
     _check(load().ia_rcp_check(x.data_ptr(), y.data_ptr(), int(x.numel()), _stream_ptr(stream)))
 
 
-def ia_test_limits(handle: int, budget: int = 0) -> None:
-    _check(load().ia_test_limits(handle, int(budget)))
+def ia_test_limits(handle: int, budget: int = 0, reserve_rounds: int = -1) -> None:
+    _check(load().ia_test_limits(handle, int(budget), int(reserve_rounds)))
 
 
 def ia_test_tail(handle: int, queue: "Queue | None" = None) -> tuple:

@@ -118,9 +118,12 @@ constexpr int LOCAL_QUANTUM = 16;
 constexpr int HARD_HOLD = 64;  // attempts of a warp without integer products after one that could not use them
 constexpr int WARP_HOLD = 64;  // attempts in warp mode between looks for records
 // Reserved tail SMs serve trajectories past the slice budget while the bulk still runs. Below this many
-// trajectories per lane the bulk is over before one can get there (131,072 attempts, over 5 s), and the
-// reserved SMs would only run the lane phase in batches; such launches reserve none.
-constexpr long long RESERVE_MIN_ROUNDS = 8;
+// trajectories per lane they mostly run the lane phase in batches, and such launches reserve none: a rule of
+// thumb from head-on runs at 1.5 uK (mean 9,000 attempts, longest 10^6; without and with 32 reserved SMs
+// 40,000 take 7.4 and 7.3 s, 100,000 7.1 and 7.6 s). It holds only where the caller leaves the number of SMs to
+// the library and the previous part of a batch left no trajectory in group mode, which would have to wait for
+// the lane phase.
+constexpr int RESERVE_MIN_ROUNDS = 8;
 
 __device__ __forceinline__ unsigned long long global_ns()
 {
@@ -1193,10 +1196,11 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
                                                        unsigned* __restrict__ ready, Susp* __restrict__ susp,
                                                        long long cap, int refill, int budget, int tail_sms,
                                                        int wait_ok, int pair, int tail_warps, int local_ok,
-                                                       int num_sms)
+                                                       int num_sms, int reserve_rounds)
 {
     __shared__ int role;     // 0 lane phase first, 1 tail worker, 2 surplus block on a reserved SM
     __shared__ int sm_rank;  // blocks of this SM that started before this one
+    __shared__ int n_res;    // SMs reserved for the tail
     // buffers of the paired tail, or the warps' records of local trajectories (never both in one launch)
     constexpr int PAIRS = G == 6 ? BLOCK / 64 : 1;
     constexpr size_t LOC_BYTES = (size_t)(BLOCK / 32) * LOCAL_MAX * sizeof(Susp);
@@ -1223,12 +1227,13 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
                 for (int l = 0; l < 32; ++l) pair_sh[k].seq_h[l] = pair_sh[k].seq_c[l] = 0ull;
         atomicCAS(&ctr->t_start, 0ull, global_ns());
         const bool reserve = budget > 0 && tail_sms > 0 &&
-                             !(local_ok && n_virt < RESERVE_MIN_ROUNDS * 32 * (long long)total_warps);
+                             !(local_ok && n_tc == 0 && n_virt < 32ll * reserve_rounds * (long long)total_warps);
         unsigned smid, rank = 0u;
         asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
         if (smid < (unsigned)MAX_TAIL_SMS) rank = atomicAdd(&ctr->sm_claim[smid], 1u);
         role = reserve && smid < (unsigned)tail_sms && smid < (unsigned)MAX_TAIL_SMS ? (rank == 0u ? 1 : 2) : 0;
-        if (blockIdx.x == 0) ctr->reserved = reserve ? (unsigned long long)tail_sms : 0ull;
+        n_res = reserve ? tail_sms : 0;
+        if (blockIdx.x == 0) ctr->reserved = (unsigned long long)n_res;
         sm_rank = (int)rank;
     }
     __syncthreads();
@@ -1238,11 +1243,12 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
     // busy, so trajectories are spread before warps are filled: up to a batch of groups on one warp of every
     // sub-partition, a batch per warp, full warps on one warp per sub-partition, then on all. (us per attempt
     // with 608 sub-partitions: 1 or 608 trajectories 5.8 and 6.1, 1,024 7.7 -- one per warp on two warps of a sub-partition
-    // 8.8 -- 3,040 7.7, 6,080 11.3, 19,456 22.8, 38,912 40.2.)
+    // 8.8 -- 3,040 7.7, 6,080 11.3, 19,456 22.8, 38,912 40.2.) Reserved SMs are not counted: their workers may be
+    // busy with the tail.
     int share = 32;
     if (local_ok) {
         constexpr int NG = 32 / G;
-        const long long sub = 4ll * num_sms, tw = (long long)total_warps;
+        const long long sub = 4ll * (num_sms - n_res), tw = (long long)total_warps * (num_sms - n_res) / num_sms;
         const bool one_per_sub = sub < tw && (n_virt <= NG * sub || (n_virt > NG * tw && n_virt <= 32 * sub));
         const long long warps = one_per_sub ? sub : tw;
         if (n_virt <= 32 * warps) share = (int)((n_virt + warps - 1) / warps);
@@ -1279,11 +1285,12 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
                 owes = false;
             }
             const int rc = tail_phase<G>(tab, ic, out, susp, ready, ctr, cap, wait_ok != 0, total_warps, part, n_tc,
-                                         r == 1 ? n_virt : 0, !part.last, loc, alive, more ? (budget >> 10) + 1 : -1);
+                                         r == 1 && share > 0 ? n_virt : 0, !part.last, loc, alive,
+                                         more ? (budget >> 10) + 1 : -1);
             if (rc == 0) break;
             if (rc == 1) {
                 n_loc = lane_phase(tab, n_sys, ic, out, part, n_virt, n_carry, ctr, ready, susp, cap, refill, budget,
-                                   true, loc, 32);
+                                   true, loc, share);
                 alive = (1u << n_loc) - 1u;
             }
         }
@@ -1664,6 +1671,7 @@ struct ia_system {
     size_t adj_scratch_bytes;
     int num_sms;
     int default_budget;       // slice budget of launches that leave it to the library
+    int reserve_rounds;       // trajectories per lane from which they reserve SMs
 };
 
 struct ia_graph {
@@ -1828,6 +1836,7 @@ struct Resolved {
     long long cap;  // suspend records
     size_t bytes;   // scratch bytes
     bool default_budget;  // the caller left slice_budget to the library
+    bool default_sms;     // ... tail_sms
 };
 
 constexpr int DEFAULT_BUDGET = 131072;
@@ -1839,6 +1848,7 @@ int resolve(int64_t n, const ia_launch_opts* opts, Resolved& r)
     if (opts) r.o = *opts;
     ia_launch_opts& o = r.o;
     if (o.kernel != IA_KERNEL_PLAIN && o.kernel != IA_KERNEL_PERSISTENT) return IA_ERR_INVALID_ARG;
+    r.default_sms = o.tail_sms == 0;
     if (o.tail_sms == 0) o.tail_sms = DEFAULT_TAIL_SMS;
     if (o.tail_sms < -1 || o.tail_sms > MAX_TAIL_SMS) return IA_ERR_INVALID_ARG;
     if (o.refill == 0) o.refill = 1;
@@ -1885,6 +1895,7 @@ struct SchedCfg {
     const void* fn;
     int block, grid, resident, budget, wait_ok, tail_sms, pair, refill, tail_warps;
     int local_ok;  // group mode for what the lane phase leaves (LOCAL_MAX)
+    int reserve_rounds;
 };
 
 int sched_config(const ia_system* sys, const Resolved& r, SchedCfg& c)
@@ -1918,6 +1929,7 @@ int sched_config(const ia_system* sys, const Resolved& r, SchedCfg& c)
     c.refill = o.refill;
     // an explicit slice budget says when trajectories move to group mode: nothing moves before it
     c.local_ok = (r.default_budget && c.wait_ok && !c.pair) ? 1 : 0;
+    c.reserve_rounds = r.default_sms ? sys->reserve_rounds : 0;
     c.tail_warps = o.tail_warps == 0 ? std::min(TAIL_WARPS, c.block / 32) : o.tail_warps;
     if (c.tail_warps < 1 || c.tail_warps > MAX_TAIL_WARPS || c.tail_warps > c.block / 32) return IA_ERR_INVALID_ARG;
     return IA_OK;
@@ -1934,11 +1946,12 @@ int launch_sched(const ia_system* sys, const SchedCfg& c, const Resolved& r, IcP
     long long cap = r.cap;
     int refill = c.refill, budget = c.budget, tail_sms = c.tail_sms, wait_ok = c.wait_ok, pair = c.pair;
     int tail_warps = c.tail_warps, local_ok = c.local_ok && part.last && !part.lane_only, num_sms = sys->num_sms;
+    int reserve_rounds = c.reserve_rounds;
     int n_sys = sys->n_sys;
     const SysDev* tab = sys->d_tab;
     void* args[] = {(void*)&tab, (void*)&n_sys, (void*)&icp, (void*)&op, (void*)&part, (void*)&ctr, (void*)&ready,
                     (void*)&susp, (void*)&cap, (void*)&refill, (void*)&budget, (void*)&tail_sms, (void*)&wait_ok,
-                    (void*)&pair, (void*)&tail_warps, (void*)&local_ok, (void*)&num_sms};
+                    (void*)&pair, (void*)&tail_warps, (void*)&local_ok, (void*)&num_sms, (void*)&reserve_rounds};
     cudaError_t e;
     if (wait_ok)
         e = cudaLaunchCooperativeKernel(c.fn, dim3(c.grid), dim3(c.block), args, 0, st);
@@ -2018,6 +2031,7 @@ int ia_system_create(const ia_system_desc* desc, int32_t n_sys, ia_system** out)
     s->adj_scratch_bytes = 0;
     s->num_sms = prop.multiProcessorCount;
     s->default_budget = DEFAULT_BUDGET;
+    s->reserve_rounds = RESERVE_MIN_ROUNDS;
     if (cudaMalloc(&s->d_tab, sizeof(SysDev) * (size_t)n_sys) != cudaSuccess ||
         cudaMemcpy(s->d_tab, host, sizeof(SysDev) * (size_t)n_sys, cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaFree(s->d_tab);
@@ -2458,7 +2472,7 @@ int ia_autotune(ia_system* sys, const ia_ic_soa* ic, int64_t n, int32_t attempt_
         int grid = resident * sys->num_sms;
         long long nn_ = (long long)n;
         int refill = cd.refill, budget = attempt_cap, tail_sms = 0, wait_ok = 0, pair = 0, n_sys = sys->n_sys;
-        int tail_warps = TAIL_WARPS, local_ok = 0, num_sms = sys->num_sms;
+        int tail_warps = TAIL_WARPS, local_ok = 0, num_sms = sys->num_sms, reserve_rounds = 0;
         long long capv = cap;
         const SysDev* tab = sys->d_tab;
         Part part = single_part(nn_);
@@ -2466,7 +2480,7 @@ int ia_autotune(ia_system* sys, const ia_ic_soa* ic, int64_t n, int32_t attempt_
         void* args[] = {(void*)&tab, (void*)&n_sys, (void*)&icp, (void*)&op, (void*)&part, (void*)&ctr,
                         (void*)&ready, (void*)&susp, (void*)&capv, (void*)&refill, (void*)&budget,
                         (void*)&tail_sms, (void*)&wait_ok, (void*)&pair, (void*)&tail_warps, (void*)&local_ok,
-                        (void*)&num_sms};
+                        (void*)&num_sms, (void*)&reserve_rounds};
         if (cudaMemsetAsync(scr, 0, SCRATCH_HEAD + ready_bytes(cap), st) != cudaSuccess) rc = IA_ERR_CUDA;
         cudaEventRecord(e0, st);
         // budget > 0 with no tail workers: the kernel stops every trajectory at the cap
@@ -2701,10 +2715,11 @@ int ia_launch_phases(ia_system* sys, const void* scratch, double* lane_ms, doubl
     return IA_OK;
 }
 
-int ia_test_limits(ia_system* sys, int32_t budget)
+int ia_test_limits(ia_system* sys, int32_t budget, int32_t reserve_rounds)
 {
-    if (!sys || budget < 0) return IA_ERR_INVALID_ARG;
+    if (!sys || budget < 0 || reserve_rounds < -1 || reserve_rounds > (1 << 20)) return IA_ERR_INVALID_ARG;
     sys->default_budget = budget ? budget : DEFAULT_BUDGET;
+    sys->reserve_rounds = reserve_rounds < 0 ? RESERVE_MIN_ROUNDS : reserve_rounds;
     return IA_OK;
 }
 

@@ -541,6 +541,15 @@ int ia_test_tail(const ia_system* sys, const ia_queue* q, int64_t* records, int6
  */
 int ia_rcp_check(const double* x, double* y, int64_t n, void* stream);
 
+/*
+ * Test hook (no counterpart in the paper): the integer forms of op 0: a[i] b[i] (integrator), op 1:
+ * sqrt(a[i]), op 2: a[i] / b[i], b[i] > 0 (sampler), which are meant to be the correctly rounded ones.
+ * general[i] = 1 where the product leaves its operands to the FP64 unit (y[i] has no meaning then).
+ * Device arrays of n elements. Asynchronous.
+ */
+int ia_rounding_check(int32_t op, const double* a, const double* b, double* y, int32_t* general, int64_t n,
+                      void* stream);
+
 /* Static description of a return code (never NULL). */
 const char* ia_error_string(int code);
 

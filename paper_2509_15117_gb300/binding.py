@@ -35,7 +35,7 @@ EXPORTED = ("ia_system_create", "ia_system_destroy", "ia_system_count", "ia_scra
             "ia_adjoint_scratch_bytes", "ia_launch_adjoint", "ia_philox4x64", "ia_sample_ics", "ia_fp64_peak",
             "ia_rcp_check", "ia_error_string", "ia_version", "ia_queue_create", "ia_queue_launch",
             "ia_queue_reset", "ia_queue_state", "ia_queue_phases", "ia_queue_destroy", "ia_static_phases",
-            "ia_test_limits", "ia_test_tail")
+            "ia_test_limits", "ia_test_tail", "ia_rounding_check")
 
 IA_SAMPLE_HEAD_ON = 0
 IA_SAMPLE_SPHERE = 1
@@ -241,6 +241,9 @@ def load(build_if_missing: bool = True):
     L.ia_reserve.restype = ctypes.c_int
     L.ia_rcp_check.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
     L.ia_rcp_check.restype = ctypes.c_int
+    L.ia_rounding_check.argtypes = [ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
+                                    ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
+    L.ia_rounding_check.restype = ctypes.c_int
     L.ia_test_limits.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32]
     L.ia_test_limits.restype = ctypes.c_int
     L.ia_test_tail.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.POINTER(ctypes.c_int64),
@@ -410,6 +413,17 @@ def ia_rcp_check(x, y, stream=None) -> None:
     _tensor(x, "x", torch.float64, (None,))
     _tensor(y, "y", torch.float64, (x.shape[0],))
     _check(load().ia_rcp_check(x.data_ptr(), y.data_ptr(), int(x.numel()), _stream_ptr(stream)))
+
+
+def ia_rounding_check(op: int, a, b, y, general, stream=None) -> None:
+    import torch
+    _tensor(a, "a", torch.float64, (None,))
+    n = int(a.shape[0])
+    _tensor(b, "b", torch.float64, (n,))
+    _tensor(y, "y", torch.float64, (n,))
+    _tensor(general, "general", torch.int32, (n,))
+    _check(load().ia_rounding_check(int(op), a.data_ptr(), b.data_ptr(), y.data_ptr(), general.data_ptr(), n,
+                                    _stream_ptr(stream)))
 
 
 def ia_test_limits(handle: int, budget: int = 0, reserve_rounds: int = -1) -> None:

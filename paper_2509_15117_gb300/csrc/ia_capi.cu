@@ -1654,6 +1654,17 @@ __global__ void k_rcp_check(const double* x, double* y, long long n)
     if (i < n) y[i] = rcp_nr(x[i]);
 }
 
+__global__ void k_rounding_check(int op, const double* a, const double* b, double* y, int* general, long long n)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    bool bad = false;
+    if (op == 0) y[i] = soft_mul(a[i], b[i], bad);
+    else if (op == 1) y[i] = ia_sample::sqrt_rn(a[i]);
+    else y[i] = ia_sample::ordinary(b[i]) ? ia_sample::div_rn(a[i], b[i], ia_sample::fx_rcp(b[i])) : a[i] / b[i];
+    general[i] = bad ? 1 : 0;
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
@@ -2812,6 +2823,20 @@ int ia_rcp_check(const double* x, double* y, int64_t n, void* stream)
     if (!aligned8(x) || !aligned8(y)) return IA_ERR_ALIGNMENT;
     const long long blocks = (n + 255) / 256;
     k_rcp_check<<<(unsigned)blocks, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(x, y, (long long)n);
+    return cudaGetLastError() == cudaSuccess ? IA_OK : IA_ERR_CUDA;
+}
+
+int ia_rounding_check(int32_t op, const double* a, const double* b, double* y, int32_t* general, int64_t n,
+                      void* stream)
+{
+    if (op < 0 || op > 2 || !a || !b || !y || !general || n < 0) return IA_ERR_INVALID_ARG;
+    if (n == 0) return IA_OK;
+    if (!aligned8(a) || !aligned8(b) || !aligned8(y) || (reinterpret_cast<uintptr_t>(general) & 3u) != 0)
+        return IA_ERR_ALIGNMENT;
+    const long long blocks = (n + 255) / 256;
+    if (blocks > 0x7fffffffLL) return IA_ERR_TOO_LARGE;
+    k_rounding_check<<<(unsigned)blocks, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(op, a, b, y, general,
+                                                                                           (long long)n);
     return cudaGetLastError() == cudaSuccess ? IA_OK : IA_ERR_CUDA;
 }
 

@@ -351,8 +351,9 @@ int ia_graph_destroy(ia_graph* graph);
  * with CUDA events on `stream`, twice (interleaved with the other candidates; the shorter time counts);
  * every candidate does the same arithmetic, so the fastest has the highest lane-phase throughput.
  * Candidates within 1 % of the fastest count as equal, and among them the smallest refill grain wins
- * (then the fastest): in the sample every trajectory stops at the same cap, which hides what a lazier
- * refill costs in a batch of spread lengths.
+ * (then a block of at least 128 threads, whose reserved SMs hold four tail warps, then the fastest): in the
+ * sample every trajectory stops at the same cap, which hides what a lazier refill costs in a batch of
+ * spread lengths, and none reaches the tail.
  * Writes the winner into *best (other fields copied from *base, which may be NULL) and its time in
  * *best_ms. Synchronous. attempt_cap: 64..1048576.
  */
@@ -534,6 +535,13 @@ int ia_test_limits(ia_system* sys, int32_t budget, int32_t reserve_rounds);
  * used up), and the SMs that its latest launch reserved for the tail. Synchronous.
  */
 int ia_test_tail(const ia_system* sys, const ia_queue* q, int64_t* records, int64_t* reserved);
+
+/*
+ * Test hook (no counterpart in the paper): the options that ia_autotune picks when its n = 9 candidates --
+ * (block, regs_variant, refill) = (128, 1, 1), (128, 1, 4), (128, 1, 16), (64, 1, 1), (64, 1, 4),
+ * (256, 1, 1), (256, 1, 4), (128, 3, 1), (128, 3, 4) -- took ms[0..8]. No CUDA call.
+ */
+int ia_test_autotune_pick(const double* ms, int32_t n, int32_t* block, int32_t* regs_variant, int32_t* refill);
 
 /*
  * Test hook (no counterpart in the paper): y[i] = 1/x[i] computed as the integrator computes 1/r^2

@@ -35,7 +35,7 @@ EXPORTED = ("ia_system_create", "ia_system_destroy", "ia_system_count", "ia_scra
             "ia_adjoint_scratch_bytes", "ia_launch_adjoint", "ia_philox4x64", "ia_sample_ics", "ia_fp64_peak",
             "ia_rcp_check", "ia_error_string", "ia_version", "ia_queue_create", "ia_queue_launch",
             "ia_queue_reset", "ia_queue_state", "ia_queue_phases", "ia_queue_destroy", "ia_static_phases",
-            "ia_test_limits", "ia_test_tail", "ia_rounding_check")
+            "ia_test_limits", "ia_test_tail", "ia_rounding_check", "ia_test_autotune_pick")
 
 IA_SAMPLE_HEAD_ON = 0
 IA_SAMPLE_SPHERE = 1
@@ -241,6 +241,9 @@ def load(build_if_missing: bool = True):
     L.ia_reserve.restype = ctypes.c_int
     L.ia_rcp_check.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
     L.ia_rcp_check.restype = ctypes.c_int
+    L.ia_test_autotune_pick.argtypes = [P(ctypes.c_double), ctypes.c_int32, P(ctypes.c_int32), P(ctypes.c_int32),
+                                        P(ctypes.c_int32)]
+    L.ia_test_autotune_pick.restype = ctypes.c_int
     L.ia_rounding_check.argtypes = [ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                     ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
     L.ia_rounding_check.restype = ctypes.c_int
@@ -424,6 +427,13 @@ def ia_rounding_check(op: int, a, b, y, general, stream=None) -> None:
     _tensor(general, "general", torch.int32, (n,))
     _check(load().ia_rounding_check(int(op), a.data_ptr(), b.data_ptr(), y.data_ptr(), general.data_ptr(), n,
                                     _stream_ptr(stream)))
+
+
+def ia_test_autotune_pick(ms) -> tuple:
+    """(block, regs_variant, refill) that ia_autotune picks for these nine times; see ionatom.h."""
+    r = [ctypes.c_int32() for _ in range(3)]
+    _check(load().ia_test_autotune_pick((ctypes.c_double * len(ms))(*ms), len(ms), *map(ctypes.byref, r)))
+    return tuple(v.value for v in r)
 
 
 def ia_test_limits(handle: int, budget: int = 0, reserve_rounds: int = -1) -> None:

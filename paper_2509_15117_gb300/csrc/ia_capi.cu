@@ -2420,6 +2420,47 @@ int ia_graph_destroy(ia_graph* graph)
 // ---------------------------------------------------------------------------------------------
 // Autotuner of the lane phase
 
+namespace {
+// Candidates of the autotuner: threads per block, minimum resident blocks per SM, refill.
+struct TuneCand {
+    int block, minb, refill;
+};
+const TuneCand tune_cands[] = {{128, 1, 1}, {128, 1, 4}, {128, 1, 16}, {64, 1, 1}, {64, 1, 4},
+                               {256, 1, 1}, {256, 1, 4}, {128, 3, 1}, {128, 3, 4}};
+constexpr int TUNE_CANDS = (int)(sizeof(tune_cands) / sizeof(tune_cands[0]));
+
+// Candidates within 1 % of the fastest are treated as equal. The smallest refill among them wins: the sample's
+// trajectories all stop at the same cap, so lanes fall idle together and a lazier refill costs nothing there;
+// in a whole batch lengths spread, and refilling each lane at once keeps warps fuller. Then a block that fills
+// a reserved SM's four sub-partitions with tail warps, which the sample does not see: the blocks of one
+// register budget take 277-281 ms on the species x energy sample, in an order that changes from run to run, but
+// the sweep in 20 parts runs at 334, 330 and 275 thousand trajectories/s with blocks of 128, 256 and 64
+// threads. Then the fastest.
+int tune_pick(const double* ms)
+{
+    int w = 0;
+    for (int c = 1; c < TUNE_CANDS; ++c) w = ms[c] < ms[w] ? c : w;
+    const double line = ms[w] * 1.01;
+    for (int c = 0; c < TUNE_CANDS; ++c) {
+        if (!(ms[c] <= line)) continue;
+        const TuneCand &a = tune_cands[c], &b = tune_cands[w];
+        const bool fa = a.block >= 32 * TAIL_WARPS, fb = b.block >= 32 * TAIL_WARPS;
+        if (a.refill != b.refill ? a.refill < b.refill : (fa != fb ? fa : ms[c] < ms[w])) w = c;
+    }
+    return w;
+}
+}  // namespace
+
+int ia_test_autotune_pick(const double* ms, int32_t n, int32_t* block, int32_t* regs_variant, int32_t* refill)
+{
+    if (!ms || n != TUNE_CANDS || !block || !regs_variant || !refill) return IA_ERR_INVALID_ARG;
+    const TuneCand w = tune_cands[tune_pick(ms)];
+    *block = w.block;
+    *regs_variant = w.minb;
+    *refill = w.refill;
+    return IA_OK;
+}
+
 int ia_autotune(ia_system* sys, const ia_ic_soa* ic, int64_t n, int32_t attempt_cap, const ia_launch_opts* base,
                 ia_launch_opts* best, double* best_ms, void* stream)
 {
@@ -2460,20 +2501,17 @@ int ia_autotune(ia_system* sys, const ia_ic_soa* ic, int64_t n, int32_t attempt_
     Counters* ctr = reinterpret_cast<Counters*>(scr);
     unsigned* ready = reinterpret_cast<unsigned*>(scr + SCRATCH_HEAD);
     Susp* susp = reinterpret_cast<Susp*>(scr + SCRATCH_HEAD + ready_bytes(cap));
-    struct Cand { int block, minb, refill; };
-    const Cand cands[] = {{128, 1, 1}, {128, 1, 4}, {128, 1, 16}, {64, 1, 1}, {64, 1, 4},
-                          {256, 1, 1}, {256, 1, 4}, {128, 3, 1}, {128, 3, 4}};
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     int rc = IA_OK;
-    constexpr int NC = (int)(sizeof(cands) / sizeof(cands[0]));
+    constexpr int NC = TUNE_CANDS;
     constexpr int PASSES = 2;  // every candidate timed twice, interleaved; its time is the shorter
     double cand_t[NC];
     for (int c = 0; c < NC; ++c) cand_t[c] = 1e300;
     for (int it = -1; it < PASSES * NC && rc == IA_OK; ++it) {
         const int c = it < 0 ? 0 : it % NC;  // it = -1: warm-up of the first candidate
-        const Cand cd = cands[c];
+        const TuneCand cd = tune_cands[c];
         const void* fn = sched_fn(cd.block, cd.minb, 6);
         int resident = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, fn, cd.block, 0) != cudaSuccess || resident <= 0) {
@@ -2502,22 +2540,9 @@ int ia_autotune(ia_system* sys, const ia_ic_soa* ic, int64_t n, int32_t attempt_
         if (rc == IA_OK) cudaEventElapsedTime(&ms, e0, e1);
         if (it >= 0 && rc == IA_OK && ms < cand_t[c]) cand_t[c] = ms;
     }
-    // Candidates within 1 % of the fastest are treated as equal, and the smallest refill among them
-    // wins (then the fastest). The sample's trajectories all stop at the same cap, so lanes fall idle
-    // together and a lazier refill costs nothing there; in a whole batch lengths spread, and refilling
-    // each lane at once keeps warps fuller.
-    double best_t = 1e300;
-    for (int c = 0; c < NC; ++c) best_t = cand_t[c] < best_t ? cand_t[c] : best_t;
-    Cand win = cands[0];
-    double win_t = 1e300;
-    for (int c = 0; c < NC; ++c) {
-        if (cand_t[c] > best_t * 1.01) continue;
-        if (win_t == 1e300 || cands[c].refill < win.refill || (cands[c].refill == win.refill && cand_t[c] < win_t)) {
-            win = cands[c];
-            win_t = cand_t[c];
-        }
-    }
-    best_t = win_t;
+    const int pick = tune_pick(cand_t);
+    const TuneCand win = tune_cands[pick];
+    const double best_t = cand_t[pick];
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaFree(obuf);

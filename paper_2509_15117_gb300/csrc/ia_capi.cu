@@ -100,21 +100,22 @@ constexpr int MAX_TAIL_WARPS = 8;
 // Group mode for what the lane phase leaves (launches with the default slice budget): once the queue is
 // empty, a warp that holds at most LOCAL_MAX trajectories writes them to its records in shared memory and
 // advances them in group mode, 32 / G at a time, all of them in turns of LOCAL_QUANTUM attempts. An FP64
-// instruction costs a sub-partition the same time for 1 lane as for 32, so an attempt costs a warp about
-// 37,000 cycles in lane mode and 13,000 per batch of five in group mode: three batches, 15 trajectories,
-// are the break-even. The same holds for a batch that is small from the start (see `share` in k_sched).
+// instruction costs a sub-partition the same time for 1 lane as for 32: with one warp on it an attempt takes
+// 23.4 us in lane mode and 7.4 per batch of five in group mode, with two 33.8 and 11.2. Three batches, 15
+// trajectories, are the break-even. The same holds for a batch that is small from the start (see `share` in
+// k_sched).
 // Against lane mode to the end: one Rb trajectory of 8,192 attempts 128 -> 64 ms, 1,024 of up to 32,768
 // attempts 1,212 -> 321 ms, 50,000 thermal ones of up to 8,192 243 -> 94 ms, the 40-system sweep of 67,240
 // 324 -> 309 ms; 262,144 trajectories of one length, which end together, 239 -> 241 ms.
 // The slice budget holds for them too: while a warp has more than one batch, those past the budget go to
 // suspend records, and idle warps take them (twelve neighbours in the queue of 40,000 trajectories, 10^6 attempts
 // each, which one warp would otherwise carry to their end: 17.6 -> 8.9 s).
-// A warp's last trajectory goes on in warp mode: 5.8 us per attempt, 7.7 in group mode, about 20 in lane mode.
-// The line at 15, measured with the integer products in lane mode (ms at 10 / 15 / 20: thermal 93.8 / 88.8 /
-// 85.0, sweep 280 / 275 / 290, the sweep in four parts of up to 32,768 attempts 745 / 645 / 626, mixed graph
-// 350 / 334 / 340, 262,144 of one length 218.5 / 218.5 / 223.6).
+// A warp's last trajectory goes on in warp mode: 5.7 us per attempt, 7.4 in group mode, about 20 in lane mode.
+// The line at 15, measured (ms at 10 / 15 / 20, two runs each, which differ by up to 5 %: thermal 93 / 88 / 87,
+// sweep 284 / 282 / 286, the sweep in four parts of up to 32,768 attempts 712 / 635 / 636, mixed graph 346 / 331 /
+// 343, 262,144 of one length 219 / 218.5 / 223).
 constexpr int LOCAL_MAX = 15;
-constexpr int LOCAL_QUANTUM = 16;
+constexpr int LOCAL_QUANTUM = 16;  // attempts in a round of group mode, and in a turn of local trajectories
 constexpr int HARD_HOLD = 64;  // attempts of a warp without integer products after one that could not use them
 constexpr int WARP_HOLD = 64;  // attempts in warp mode between looks for records
 // Reserved tail SMs serve trajectories past the slice budget while the bulk still runs. Below this many
@@ -375,22 +376,21 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
     int sid = 0;
     bool active = false, drained = false;
     unsigned idle_spins = 0;
-    unsigned claim_skip = 0;  // iterations without a claim attempt while other groups of the warp run
+    unsigned claim_skip = 0;  // rounds without a claim attempt while other groups of the warp run
     bool yield_room = true;   // false once a yield found the record area full (warp-uniform)
     // local records: unfinished ones, those not held by a group now, this group's (-1: none), the first of
-    // the next turn, attempts left of this turn (all but lslot warp-uniform)
+    // the next turn (all but lslot warp-uniform)
     unsigned lalive = alive, lpend = lalive;
-    int lslot = -1, lnext = 0, lturn = 0;
+    int lslot = -1, lnext = 0;
     // warp mode (G = 6): while the warp has a single trajectory, every group holds a copy of it and group 0
-    // answers for it; left every WARP_HOLD attempts to look for records
+    // answers for it; left after WARP_HOLD attempts to look for records
     bool wmode = false;
-    int hold = 0;
     SysDev P;                 // the fields that an attempt needs, in registers (see group_sys)
     GroupSys gs;
     int sid_in_regs = -1;
     const WarpIdx wi = warp_idx(gl.base / G);
     for (;;) {
-        if (G == 6 && wmode && --hold < 0) {
+        if (G == 6 && wmode) {
             wmode = false;
             if (gl.base != 0) {
                 if (active) lslot = -1;  // (a finished one keeps its slot, to be cleared below)
@@ -398,12 +398,11 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
             }
             claim_skip = 0;
         }
-        if (!wmode) {
         if (lalive) {
             const unsigned done = __reduce_or_sync(FULL, lslot >= 0 && !active ? 1u << lslot : 0u);
             lalive &= ~done;
             if (!active) lslot = -1;
-            if (lpend && (done || --lturn < 0)) {
+            if (lpend) {
                 // next turn: the groups leave their trajectories and take the next ones in cyclic order
                 if (active && gl.c < G) {
                     Susp* r = loc + lslot;
@@ -451,7 +450,6 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
                     const int nxt = first + take >= n_al ? first + take - n_al : first + take;
                     lnext = (int)__fns(lalive, 0, nxt + 1);
                 }
-                lturn = LOCAL_QUANTUM;
                 __syncwarp();
             }
         }
@@ -504,13 +502,13 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
         bool poll = needy != 0u;
         if (poll && claim_skip > 0 && __any_sync(FULL, active)) {
             // an idle group polls the record counters (global atomics, microseconds) only every
-            // CLAIM_BACKOFF attempts while its warp still runs other trajectories
+            // CLAIM_BACKOFF attempts (in rounds of LOCAL_QUANTUM) while its warp still runs other trajectories
             --claim_skip;
             poll = false;
         }
         if (poll) {
             // One group claims at a time, so that records published together go to several idle warps (five
-            // in one warp step at 7.7 us per attempt, one at 5.8); its first lane does, for the whole warp.
+            // in one warp step at 7.4 us per attempt, one at 5.7); its first lane does, for the whole warp.
             const int asker = __ffs((int)needy) - 1;
             const bool ask = (int)(threadIdx.x & 31) == asker;
             int got = 0;
@@ -555,7 +553,7 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
             }
             got = __shfl_sync(FULL, got, asker);
             k = __shfl_sync(FULL, k, asker);
-            claim_skip = CLAIM_BACKOFF;
+            claim_skip = CLAIM_BACKOFF / LOCAL_QUANTUM;
             if (need) {
                 if ((got == 1 || got == 4) && gl.base == asker) {
                     // written by another SM during this launch (or by the previous launch): read through L2
@@ -608,9 +606,7 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
                 lslot = __shfl_sync(FULL, lslot, b);
                 active = true;
                 wmode = true;
-                hold = WARP_HOLD;
             }
-        }
         }
 
         if (sid != sid_in_regs) {
@@ -621,74 +617,16 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
             gs = group_sys(tab[sid], gl.c);
             sid_in_regs = sid;
         }
+        // A round: attempts until something ends, at most WARP_HOLD or LOCAL_QUANTUM of them. Turns, records and the
+        // end of the part are looked at between rounds, not between attempts (us per attempt, looked at between
+        // attempts -> between rounds: one trajectory 5.85 -> 5.70, 1,024 7.8 -> 7.4, 7,001 15.4 -> 14.6).
         uint32_t st = 0xffffffffu;
-        if (active) st = attempt_begin(P, S);
-        const double h = S.h, t = S.t;
-        double a3, a4, a5, a6, a7, xn, vn, r2new, rd;
+        double h, t, a3, a4, a5, a6, a7, xn, vn, r2new, rd;
         bool accept, finite;
         ErrMeas em;
-        if (G == 6 && wmode) {
-            WarpStep E;
-            GroupLane<6> g6;
-            g6.base = gl.base; g6.c = gl.c; g6.comp = gl.comp;
-            warp_step(P, g6, gs, wi, x, v, a1, h, t, S.phi0, E);
-            a3 = E.a3; a4 = E.a4; a5 = E.a5; a6 = E.a6; a7 = E.a7; xn = E.xn; vn = E.vn;
-            r2new = E.r2new; rd = E.rd; accept = E.accept; finite = E.finite; em = E.em;
-        } else {
-
-        // step coefficients, spread over the group's lanes
-        Coef K;
-        K.h2 = dmul(P, h, h);
-        double cv[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int k = r * G + (gl.c < G ? gl.c : 0);
-            const int kk = k < N_COEF ? k : N_COEF - 1;
-            cv[r] = dmul(P, coef_sh()[kk], COEF_H2[kk] ? K.h2 : h);
-        }
-        {
-            double* kp = &K.c2;
-#pragma unroll
-            for (int k = 0; k < N_COEF; ++k) kp[k] = shfl(cv[k / G], gl.base + (k % G));
-        }
-        // rf phases of stages 2..6 (stage 7 shares stage 6's time), one per lane
-        const double chsel = gl.c < 4 ? cv[0] : h;
-        const double cl = cos(fma(P.Omega, dadd(P, t, chsel), S.phi0));
-        const double cs2 = shfl(cl, gl.base + 0), cs3 = shfl(cl, gl.base + 1), cs4 = shfl(cl, gl.base + 2);
-        const double cs5 = shfl(cl, gl.base + 3), cs67 = shfl(cl, gl.base + 4);
-
-        double r2, d3[3];
-        const double a2 = accel_group<G>(P, gl, gs, pos2(K, x, v), cs2, r2, d3);
-        a3 = accel_group<G>(P, gl, gs, pos3(K, x, v, a1), cs3, r2, d3);
-        a4 = accel_group<G>(P, gl, gs, pos4(K, x, v, a1, a2), cs4, r2, d3);
-        a5 = accel_group<G>(P, gl, gs, pos5(K, x, v, a1, a2, a3), cs5, r2, d3);
-        a6 = accel_group<G>(P, gl, gs, pos6(K, h, x, v, a1, a2, a3, a4), cs67, r2, d3);
-        xn = pos7(K, h, x, v, a1, a3, a4, a5);
-        double dn[3];
-        a7 = accel_group<G>(P, gl, gs, xn, cs67, r2new, dn);
-        vn = vel_new(K, v, a1, a3, a4, a5, a6);
-
-        bool okx, fx, okv, fv;
-        float rx, rv;
-        double aex, scx, aev, scv;
-        err_check(P, P.rtol, P.atol_pos, x, xn, err_x(P, K, a1, a3, a4, a5, a6), okx, fx, rx, aex, scx);
-        err_check(P, P.rtol, P.atol_vel, v, vn, err_v(P, K, a1, a3, a4, a5, a6, a7), okv, fv, rv, aev, scv);
-        const bool real = gl.c < 6;
-        const bool ok = !real || (okx && okv);
-        const bool fi = !real || (fx && fv);
-        const unsigned gmask = ((1u << G) - 1u) << gl.base;
-        accept = (__ballot_sync(FULL, !ok) & gmask) == 0;
-        finite = (__ballot_sync(FULL, !fi) & gmask) == 0;
-        em = group_err(gl.base, gl.c, real, rx, aex, scx, rv, aev, scv);
-        // radial velocity sign at the step end: d . (v_a - v_i)
-        const int j = gl.comp < 3 ? gl.comp : gl.comp - 3;
-        const double wj = dsub(P, shfl(vn, gl.base + 3 + j), shfl(vn, gl.base + j));
-        const double w0 = shfl(wj, gl.base + 0), w1 = shfl(wj, gl.base + 1), w2 = shfl(wj, gl.base + 2);
-        rd = fma(dn[0], w0, fma(dn[1], w1, dmul(P, dn[2], w2)));
-        }
-
         int res = 0;  // 0 running, 1 stopped, 2 exits in this step
-        if (active) {
+        const auto decide = [&]() {
+            if (!active) return;
             if (st != 0xffffffffu) {
                 res = 1;
             } else if (!finite) {
@@ -705,6 +643,77 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
                 a1 = a7;
                 on_commit(P, S, em);
             }
+        };
+        int left = G == 6 && wmode ? WARP_HOLD : LOCAL_QUANTUM;
+        if (G == 6 && wmode) {
+            GroupLane<6> g6;
+            g6.base = gl.base; g6.c = gl.c; g6.comp = gl.comp;
+            do {
+                st = attempt_begin(P, S);
+                h = S.h; t = S.t;
+                WarpStep E;
+                warp_step(P, g6, gs, wi, x, v, a1, h, t, S.phi0, E);
+                a3 = E.a3; a4 = E.a4; a5 = E.a5; a6 = E.a6; a7 = E.a7; xn = E.xn; vn = E.vn;
+                r2new = E.r2new; rd = E.rd; accept = E.accept; finite = E.finite; em = E.em;
+                decide();
+            } while (res == 0 && --left > 0);
+        } else {
+            do {
+                st = 0xffffffffu;
+                if (active) st = attempt_begin(P, S);
+                h = S.h; t = S.t;
+
+                // step coefficients, spread over the group's lanes
+                Coef K;
+                K.h2 = dmul(P, h, h);
+                double cv[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int k = r * G + (gl.c < G ? gl.c : 0);
+                    const int kk = k < N_COEF ? k : N_COEF - 1;
+                    cv[r] = dmul(P, coef_sh()[kk], COEF_H2[kk] ? K.h2 : h);
+                }
+                {
+                    double* kp = &K.c2;
+#pragma unroll
+                    for (int k = 0; k < N_COEF; ++k) kp[k] = shfl(cv[k / G], gl.base + (k % G));
+                }
+                // rf phases of stages 2..6 (stage 7 shares stage 6's time), one per lane
+                const double chsel = gl.c < 4 ? cv[0] : h;
+                const double cl = cos(fma(P.Omega, dadd(P, t, chsel), S.phi0));
+                const double cs2 = shfl(cl, gl.base + 0), cs3 = shfl(cl, gl.base + 1), cs4 = shfl(cl, gl.base + 2);
+                const double cs5 = shfl(cl, gl.base + 3), cs67 = shfl(cl, gl.base + 4);
+
+                double r2, d3[3];
+                const double a2 = accel_group<G>(P, gl, gs, pos2(K, x, v), cs2, r2, d3);
+                a3 = accel_group<G>(P, gl, gs, pos3(K, x, v, a1), cs3, r2, d3);
+                a4 = accel_group<G>(P, gl, gs, pos4(K, x, v, a1, a2), cs4, r2, d3);
+                a5 = accel_group<G>(P, gl, gs, pos5(K, x, v, a1, a2, a3), cs5, r2, d3);
+                a6 = accel_group<G>(P, gl, gs, pos6(K, h, x, v, a1, a2, a3, a4), cs67, r2, d3);
+                xn = pos7(K, h, x, v, a1, a3, a4, a5);
+                double dn[3];
+                a7 = accel_group<G>(P, gl, gs, xn, cs67, r2new, dn);
+                vn = vel_new(K, v, a1, a3, a4, a5, a6);
+
+                bool okx, fx, okv, fv;
+                float rx, rv;
+                double aex, scx, aev, scv;
+                err_check(P, P.rtol, P.atol_pos, x, xn, err_x(P, K, a1, a3, a4, a5, a6), okx, fx, rx, aex, scx);
+                err_check(P, P.rtol, P.atol_vel, v, vn, err_v(P, K, a1, a3, a4, a5, a6, a7), okv, fv, rv, aev, scv);
+                const bool real = gl.c < 6;
+                const bool ok = !real || (okx && okv);
+                const bool fi = !real || (fx && fv);
+                const unsigned gmask = ((1u << G) - 1u) << gl.base;
+                accept = (__ballot_sync(FULL, !ok) & gmask) == 0;
+                finite = (__ballot_sync(FULL, !fi) & gmask) == 0;
+                em = group_err(gl.base, gl.c, real, rx, aex, scx, rv, aev, scv);
+                // radial velocity sign at the step end: d . (v_a - v_i)
+                const int j = gl.comp < 3 ? gl.comp : gl.comp - 3;
+                const double wj = dsub(P, shfl(vn, gl.base + 3 + j), shfl(vn, gl.base + j));
+                const double w0 = shfl(wj, gl.base + 0), w1 = shfl(wj, gl.base + 1), w2 = shfl(wj, gl.base + 2);
+                rd = fma(dn[0], w0, fma(dn[1], w1, dmul(P, dn[2], w2)));
+                decide();
+            } while (!__any_sync(FULL, res != 0) && --left > 0);
         }
         if (__any_sync(FULL, res != 0)) {
             Final fin;
@@ -738,7 +747,6 @@ __device__ __forceinline__ int tail_phase(const SysDev* __restrict__ tab, const 
             if (res != 0) {
                 if (gl.c == 0 && !(wmode && gl.base != 0)) store_result(tab[sid], ic, out, idx, tally(S), fin, true);
                 active = false;
-                hold = 0;
             }
         }
     }
@@ -1242,8 +1250,8 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
     // Share of a small batch. A warp's attempt costs its sub-partition the same time however few lanes are
     // busy, so trajectories are spread before warps are filled: up to a batch of groups on one warp of every
     // sub-partition, a batch per warp, full warps on one warp per sub-partition, then on all. (us per attempt
-    // with 608 sub-partitions: 1 or 608 trajectories 5.8 and 6.1, 1,024 7.7 -- one per warp on two warps of a sub-partition
-    // 8.8 -- 3,040 7.7, 6,080 11.3, 19,456 22.8, 38,912 40.2.) Reserved SMs are not counted: their workers may be
+    // with 608 sub-partitions: 1 or 608 trajectories 5.7 and 6.0, 1,024 7.4 -- one per warp on two warps of a sub-partition
+    // 8.8 -- 3,040 7.4, 6,080 11.2, 19,456 23.4, 38,912 33.8.) Reserved SMs are not counted: their workers may be
     // busy with the tail.
     int share = 32;
     if (local_ok) {
@@ -1271,12 +1279,9 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_sched(const SysDev* __restrict_
         // trajectories for the next part. A reserved SM's worker that finds the tail queue empty runs batches of
         // the lane phase meanwhile. (The lane-only timing runs of the autotuner leave trajectories past the
         // budget in their records.)
-        // (The empty asm keeps the two loops apart for the compiler; merged, an attempt took 2 % longer.)
         unsigned alive = (1u << n_loc) - 1u;
-#pragma unroll 1
         for (;;) {
             bool more = false;
-            asm volatile("" : "+r"(alive) : : "memory");
             if (__popc(alive) > 32 / G)
                 alive = publish_local(tab, loc, alive, 32 / G, budget, ctr, ready, susp, cap, more);
             // (budget / 1,024 turns of LOCAL_QUANTUM attempts: a look every few ms)
@@ -1891,7 +1896,9 @@ int resolve(int64_t n, const ia_launch_opts* opts, Resolved& r)
 }
 
 // Builds of the fused persistent kernel: (block, minimum resident blocks per SM, tail group size).
-// The register cap of 3 x 128-thread blocks per SM (168 registers) is the only one that does not spill.
+// The cap of 3 x 128-thread blocks per SM (168 registers) spills 2.8 KB (the others tens of bytes) and has half as
+// many warps again: 262,144 trajectories at 1 mK 219 ms in both builds, 58,368 of 2,000 attempts 104 ms against 113,
+// but the species x energy sweep, with its tail, 299 thousand trajectories/s against 334.
 const void* sched_fn(int block, int minb, int g)
 {
     if (block == 64) return (const void*)k_sched<64, 1, 6>;

@@ -1123,7 +1123,7 @@ __device__ __forceinline__ ErrMeas group_err(int base, int c, bool real, float r
 // stages 3..7, new velocity, the two error estimates, each a chain of DFMAs in the order of m -- are
 // spread over the groups, so that one instruction advances up to five chains; every value is formed by
 // the expression of the other layouts. About 140 FP64 instructions per attempt instead of group mode's 200,
-// one after the other; 5.8 us per attempt instead of 7.7 (9.7 with the system's constants loaded in every
+// one after the other; 5.7 us per attempt instead of 7.4 (9.7 with the system's constants loaded in every
 // attempt and idle groups at zero separation).
 //
 // acc holds X3..X7 on groups 0..4, aux the new velocity, position error and velocity error on groups 0..2.
@@ -1133,7 +1133,7 @@ struct WarpStep {
     ErrMeas em;
 };
 
-// Lanes that hold the coefficient of each group in each sum (i0..i4 by group), packed six bits each: a
+// Lanes that hold the coefficient of each group in each sum (i0..i4 by group), packed five bits each: a
 // lane's indices are constants of the launch, kept in two registers.
 __device__ __forceinline__ int pick5(int g, int i0, int i1, int i2, int i3, int i4)
 {

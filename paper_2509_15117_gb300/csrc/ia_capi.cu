@@ -109,7 +109,7 @@ constexpr int MAX_TAIL_WARPS = 8;
 // 324 -> 309 ms; 262,144 trajectories of one length, which end together, 239 -> 241 ms.
 // The slice budget holds for them too: while a warp has more than one batch, those past the budget go to
 // suspend records, and idle warps take them (twelve neighbours in the queue of 40,000 trajectories, 10^6 attempts
-// each, which one warp would otherwise carry to their end: 17.6 -> 8.9 s).
+// each, which one warp would otherwise carry to their end: 17.7 -> 8.7 s).
 // A warp's last trajectory goes on in warp mode: 5.7 us per attempt, 7.4 in group mode, about 20 in lane mode.
 // The line at 15, measured (ms at 10 / 15 / 20, two runs each, which differ by up to 5 %: thermal 93 / 88 / 87,
 // sweep 284 / 282 / 286, the sweep in four parts of up to 32,768 attempts 712 / 635 / 636, mixed graph 346 / 331 /
@@ -1898,7 +1898,7 @@ int resolve(int64_t n, const ia_launch_opts* opts, Resolved& r)
 // Builds of the fused persistent kernel: (block, minimum resident blocks per SM, tail group size).
 // The cap of 3 x 128-thread blocks per SM (168 registers) spills 2.8 KB (the others tens of bytes) and has half as
 // many warps again: 262,144 trajectories at 1 mK 219 ms in both builds, 58,368 of 2,000 attempts 104 ms against 113,
-// but the species x energy sweep, with its tail, 299 thousand trajectories/s against 334.
+// but the species x energy sweep, with its tail, 346 thousand trajectories/s against 364.
 const void* sched_fn(int block, int minb, int g)
 {
     if (block == 64) return (const void*)k_sched<64, 1, 6>;
@@ -2441,7 +2441,7 @@ constexpr int TUNE_CANDS = (int)(sizeof(tune_cands) / sizeof(tune_cands[0]));
 // in a whole batch lengths spread, and refilling each lane at once keeps warps fuller. Then a block that fills
 // a reserved SM's four sub-partitions with tail warps, which the sample does not see: the blocks of one
 // register budget take 277-281 ms on the species x energy sample, in an order that changes from run to run, but
-// the sweep in 20 parts runs at 334, 330 and 275 thousand trajectories/s with blocks of 128, 256 and 64
+// the sweep in 20 parts runs at 364, 359 and 277 thousand trajectories/s with blocks of 128, 256 and 64
 // threads. Then the fastest.
 int tune_pick(const double* ms)
 {
